@@ -31,8 +31,8 @@ UNITS = {
     "rrmhd_server.cu": ["--fmad=false"],
     "rrmhd_probe.cu": [],
 }
-HEADERS = ["physics_f64.cuh", "scheme_f64.cuh", "physics_tangent.cuh", "batch.h", "batch_index.cuh",
-           "engine.h"]
+HEADERS = ["fp64_int.cuh", "physics_f64.cuh", "scheme_f64.cuh", "physics_tangent.cuh", "batch.h", "batch_index.cuh",
+           "engine.h", "launch_shape.cuh"]
 
 
 def _deps():

@@ -14,9 +14,25 @@
 #pragma once
 #include <cstdint>
 
+#include "fp64_int.cuh"
+
 namespace rr {
 
 constexpr int NV = 12;
+
+// Correctly rounded a / b and sqrt(x) of the FP64 path (fp64_int.cuh).  The _call forms are
+// one shared copy of the code, for places off the innermost loops: an inline quotient is
+// ~60 instructions (1 KB), and the solvers' instruction footprint matters.
+static __device__ __noinline__ double ddiv_call(double a, double b) { return fpi::div(a, b); }
+static __device__ __noinline__ double dsqrt_call(double x) { return fpi::sqrt(x); }
+__device__ __forceinline__ float ddiv_call(float a, float b) { return a / b; }
+#ifdef RR_DIV_CALLS
+__device__ __forceinline__ double ddiv(double a, double b) { return ddiv_call(a, b); }
+__device__ __forceinline__ double dsqrt(double x) { return dsqrt_call(x); }
+#else
+__device__ __forceinline__ double ddiv(double a, double b) { return fpi::div(a, b); }
+__device__ __forceinline__ double dsqrt(double x) { return fpi::sqrt(x); }
+#endif
 
 enum Status : int {
   ST_OK = 0,
@@ -56,8 +72,8 @@ __device__ __forceinline__ void aux_of(const Params& P, const double* V, Aux& a)
   const double vx = V[1], vy = V[2], vz = V[3];
   const double Bx = V[5], By = V[6], Bz = V[7];
   a.v2 = (vx * vx + vy * vy) + vz * vz;
-  a.iW = sqrt(1.0 - a.v2);
-  a.W = 1.0 / a.iW;
+  a.iW = dsqrt(1.0 - a.v2);
+  a.W = ddiv(1.0, a.iW);
   a.vB = (vx * Bx + vy * By) + vz * Bz;
   a.B2 = (Bx * Bx + By * By) + Bz * Bz;
   a.b0 = a.W * a.vB;
@@ -88,7 +104,7 @@ __device__ __forceinline__ void prim2con(const Params& P, const double* V, doubl
   U[2] = hw * V[2] - a.b0 * a.b[1];
   U[3] = hw * V[3] - a.b0 * a.b[2];
   const double u2 = W2 * a.v2;
-  const double e1 = D * (u2 / (a.W + 1.0));
+  const double e1 = D * ddiv(u2, a.W + 1.0);
   const double e2 = (P.gfac * V[4] + a.bsq) * W2;
   U[4] = (e1 + e2) - (a.ptot + a.b0 * a.b0);
 #pragma unroll
@@ -103,14 +119,17 @@ struct M1 {
 };
 
 __device__ __forceinline__ M1 m1_coef(double E, double Fx, double Fy, double Fz) {
-  const double F2 = (Fx * Fx + Fy * Fy) + Fz * Fz;
-  double f2 = F2 / (E * E);
+  // uncontracted in every unit: the FP32-bulk unit's results must not depend on how the
+  // compiler fuses this sum with what is inlined around it
+  const double F2 = __dadd_rn(__dadd_rn(__dmul_rn(Fx, Fx), __dmul_rn(Fy, Fy)), __dmul_rn(Fz, Fz));
+  double f2 = ddiv(F2, E * E);
   if (f2 > 1.0) f2 = 1.0;
-  const double xi = (3.0 + 4.0 * f2) / (5.0 + 2.0 * sqrt(4.0 - 3.0 * f2));
+  const double xi = ddiv(3.0 + 4.0 * f2, 5.0 + 2.0 * dsqrt(4.0 - 3.0 * f2));
   M1 m;
   m.a = (0.5 * (1.0 - xi)) * E;
   m.c = 0.0;
-  if (F2 > 0.0) m.c = ((0.5 * (3.0 * xi - 1.0)) * E) / F2;
+  const double mc = ddiv((0.5 * (3.0 * xi - 1.0)) * E, F2 > 0.0 ? F2 : 1.0);
+  if (F2 > 0.0) m.c = mc;
   return m;
 }
 
@@ -122,11 +141,11 @@ __device__ __forceinline__ double m1_P(const M1& m, const double* F, int i, int 
 // Eddington tensor D_r = P_r/E_r (coefficients without the E_r factor).
 __device__ __forceinline__ void eddington(double E, const double* F, double Dr[3][3]) {
   const double F2 = (F[0] * F[0] + F[1] * F[1]) + F[2] * F[2];
-  double f2 = F2 / (E * E);
+  double f2 = ddiv(F2, E * E);
   if (f2 > 1.0) f2 = 1.0;
-  const double xi = (3.0 + 4.0 * f2) / (5.0 + 2.0 * sqrt(4.0 - 3.0 * f2));
+  const double xi = ddiv(3.0 + 4.0 * f2, 5.0 + 2.0 * dsqrt(4.0 - 3.0 * f2));
   const double a = 0.5 * (1.0 - xi);
-  const double c = (F2 > 0.0) ? (0.5 * (3.0 * xi - 1.0)) / F2 : 0.0;
+  const double c = (F2 > 0.0) ? ddiv(0.5 * (3.0 * xi - 1.0), F2) : 0.0;
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
@@ -168,53 +187,83 @@ __device__ __forceinline__ void flux(const Params& P, int d, const double* V, co
 struct C2PIn {
   double D, S[3], tau, B[3], S2, B2, SB, SB2, gm1g;
 };
-struct C2PPt {
-  int ok;
-  double x, Z, iZ, iZB, v2, W, p, f, df;
+struct C2PPt {  // the root
+  double Z, iZ, iZB, v2, W, p;
 };
 
-// FAST (the FP32-bulk form's cells): 1/Z and 1/(Z+B^2) from one division, W from
-// rsqrt; the same values to a few ulps.  Otherwise the operation order above.
-template <bool FAST = false>
-__device__ __forceinline__ void c2p_eval(const C2PIn& c, double x, C2PPt& e) {
-  e.x = x;
-  e.ok = 0;
-  if (!(x > 0.0)) return;
-  const double Z = x + c.D;
-  const double ZB = Z + c.B2;
-  double iZ, iZB;
-  if constexpr (FAST) {
-    const double q = 1.0 / (Z * ZB);
-    iZ = ZB * q;
-    iZB = Z * q;
-  } else {
-    iZ = 1.0 / Z;
-    iZB = 1.0 / ZB;
+// Newton's iteration from x > 0: the point of the last step, or false.  One loop holds the
+// one copy of the evaluation, whatever it is for (the first point, doubled until
+// admissible; Newton points, the step halved until admissible), and f and df are formed
+// only where another Newton step follows.
+// FAST (the FP32-bulk form's cells): 1/Z and 1/(Z+B^2) from one division, W from rsqrt
+// (the same values to a few ulps) and an inexact Newton step with an FP32 reciprocal of
+// df (~6e-8 relative).
+template <bool FAST>
+__device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2PPt& e) {
+  double xt = x, dx = 0.0;
+  int it = 0, k = 0;
+  for (;;) {
+    bool ok = xt > 0.0;
+    double Z, iZ, iZB, iZ2, v2;
+    if (ok) {
+      Z = xt + c.D;
+      const double ZB = Z + c.B2;
+      if constexpr (FAST) {
+        const double q = ddiv(1.0, Z * ZB);
+        iZ = ZB * q;
+        iZB = Z * q;
+      } else {
+        iZ = ddiv(1.0, Z);
+        iZB = ddiv(1.0, ZB);
+      }
+      iZ2 = iZ * iZ;
+      v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * (iZB * iZB);
+      ok = v2 < 1.0;
+    }
+    if (!ok) {
+      if (k == (it == 0 ? 200 : 60)) return false;
+      ++k;
+      if (it == 0) {
+        xt = 2.0 * xt;
+      } else {
+        dx = 0.5 * dx;
+        xt = x + dx;
+      }
+      continue;
+    }
+    x = xt;
+    const double omv2 = 1.0 - v2;
+    double W;
+    if constexpr (FAST)
+      W = rsqrt(omv2);
+    else
+      W = ddiv(1.0, dsqrt(omv2));
+    const double p = c.gm1g * (x * omv2 - c.D * ddiv(v2, W + 1.0));
+    if (it > 0 && fabs(dx) <= 1e-10 * x) {
+      e.Z = Z;
+      e.iZ = iZ;
+      e.iZB = iZB;
+      e.v2 = v2;
+      e.W = W;
+      e.p = p;
+      return true;
+    }
+    if (it == maxit) return false;
+    const double f = ((x - p) + (0.5 * c.B2) * (1.0 + v2)) - ((0.5 * c.SB2) * iZ2 + c.tau);
+    const double dv2 = (-2.0 * ((iZB * iZB) * iZB)) *
+                       (c.S2 + c.SB2 * (((3.0 * Z + 3.0 * c.B2) * Z + c.B2 * c.B2) * (iZ2 * iZ)));
+    const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
+    const double df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * (iZ2 * iZ);
+    if constexpr (FAST) {
+      const float d32 = (float)df;
+      dx = (fabsf(d32) > 1e-30f && fabsf(d32) < 1e30f) ? -f * (double)__frcp_rn(d32) : ddiv(-f, df);
+    } else {
+      dx = ddiv(-f, df);
+    }
+    xt = x + dx;
+    ++it;
+    k = 0;
   }
-  const double iZ2 = iZ * iZ;
-  const double v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * (iZB * iZB);
-  if (!(v2 < 1.0)) return;
-  const double omv2 = 1.0 - v2;
-  double W;
-  if constexpr (FAST)
-    W = rsqrt(omv2);
-  else
-    W = 1.0 / sqrt(omv2);
-  const double p = c.gm1g * (x * omv2 - c.D * (v2 / (W + 1.0)));
-  const double f = ((x - p) + (0.5 * c.B2) * (1.0 + v2)) - ((0.5 * c.SB2) * iZ2 + c.tau);
-  const double dv2 = (-2.0 * ((iZB * iZB) * iZB)) *
-                     (c.S2 + c.SB2 * (((3.0 * Z + 3.0 * c.B2) * Z + c.B2 * c.B2) * (iZ2 * iZ)));
-  const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
-  const double df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * (iZ2 * iZ);
-  e.Z = Z;
-  e.iZ = iZ;
-  e.iZB = iZB;
-  e.v2 = v2;
-  e.W = W;
-  e.p = p;
-  e.f = f;
-  e.df = df;
-  e.ok = 1;
 }
 
 // Returns a Status; V, *Zout and *Wout (the Lorentz factor; may be null) are written
@@ -245,39 +294,8 @@ static __device__ __noinline__ int con2prim(const Params& P, const double* U, do
   double x = Zguess - c.D;
   if (!(x > 0.0)) x = (c.tau > 0.0) ? c.tau : c.D;
   C2PPt e;
-  c2p_eval<FAST>(c, x, e);
-  for (int k = 0; k < 200 && !e.ok; ++k) {
-    x = 2.0 * x;
-    c2p_eval<FAST>(c, x, e);
-  }
-  if (!e.ok) return ST_C2P;
-
-  int conv = 0;
-  for (int it = 1; it <= P.c2p_maxit; ++it) {
-    double dx;
-    if constexpr (FAST) {  // inexact Newton: an FP32 reciprocal of df (~6e-8 relative)
-      const float d32 = (float)e.df;
-      dx = (fabsf(d32) > 1e-30f && fabsf(d32) < 1e30f) ? -e.f * (double)__frcp_rn(d32)
-                                                        : -e.f / e.df;
-    } else {
-      dx = -e.f / e.df;
-    }
-    C2PPt en;
-    c2p_eval<FAST>(c, x + dx, en);
-    for (int k = 0; k < 60 && !en.ok; ++k) {
-      dx = 0.5 * dx;
-      c2p_eval<FAST>(c, x + dx, en);
-    }
-    if (!en.ok) break;
-    x = en.x;
-    e = en;
-    if (fabs(dx) <= 1e-10 * x) {
-      conv = 1;
-      break;
-    }
-  }
-  if (!conv || !(e.p > 0.0)) return ST_C2P;
-  const double rho = FAST ? c.D * ((1.0 - e.v2) * e.W) : c.D / e.W;  // D/W = D (1 - v^2) W
+  if (!c2p_root<FAST>(c, x, P.c2p_maxit, e) || !(e.p > 0.0)) return ST_C2P;
+  const double rho = FAST ? c.D * ((1.0 - e.v2) * e.W) : ddiv(c.D, e.W);  // D/W = D (1 - v^2) W
   const double SBiZ = c.SB * e.iZ;
   V[0] = rho;
   V[1] = (c.S[0] + SBiZ * c.B[0]) * e.iZB;
@@ -299,33 +317,34 @@ __device__ __forceinline__ void mhd_speeds(const Params& P, int d, const double*
                                            double& lp) {
   Aux a;
   aux_of(P, V, a);
-  const double cs2 = (P.gamma * V[4]) / a.rhoh;
-  const double ca2 = a.bsq / (a.rhoh + a.bsq);
+  const double cs2 = ddiv_call(P.gamma * V[4], a.rhoh);
+  const double ca2 = ddiv_call(a.bsq, a.rhoh + a.bsq);
   const double a2 = (cs2 + ca2) - cs2 * ca2;
   const double vd = V[1 + d];
   const double den = 1.0 - a.v2 * a2;
   double disc = (a2 * (1.0 - a.v2)) * (den - (vd * vd) * (1.0 - a2));
   if (disc < 0.0) disc = 0.0;
-  const double sq = sqrt(disc);
-  lp = (vd * (1.0 - a2) + sq) / den;
-  lm = (vd * (1.0 - a2) - sq) / den;
+  const double sq = dsqrt(disc);
+  lp = ddiv_call(vd * (1.0 - a2) + sq, den);
+  lm = ddiv_call(vd * (1.0 - a2) - sq, den);
 }
 
 // Outer radiation eigenvalues l1 <= l3 (Eqs. lam1-lam3), theta between F_r and d.
 __device__ __forceinline__ void rad_speeds(int d, const double* V, double& l1, double& l3) {
   const double E = V[8];
   const double F2 = (V[9] * V[9] + V[10] * V[10]) + V[11] * V[11];
-  const double Fn = sqrt(F2);
-  double f = Fn / E;
+  const double Fn = dsqrt(F2);
+  double f = ddiv_call(Fn, E);
   if (f > 1.0) f = 1.0;
-  const double cth = (Fn > 0.0) ? V[9 + d] / Fn : 0.0;
+  const double cq = ddiv_call(V[9 + d], Fn > 0.0 ? Fn : 1.0);
+  const double cth = (Fn > 0.0) ? cq : 0.0;
   const double f2 = f * f;
-  const double s = sqrt(4.0 - 3.0 * f2);
+  const double s = dsqrt(4.0 - 3.0 * f2);
   double arg = (2.0 / 3.0) * ((4.0 - 3.0 * f2) - s) + (2.0 * (cth * cth)) * ((2.0 - f2) - s);
   if (arg < 0.0) arg = 0.0;
-  const double zeta = sqrt(arg);
-  l1 = (f * cth - zeta) / s;
-  l3 = (f * cth + zeta) / s;
+  const double zeta = dsqrt(arg);
+  l1 = ddiv_call(f * cth - zeta, s);
+  l3 = ddiv_call(f * cth + zeta, s);
 }
 
 __device__ __forceinline__ double signal_speed(const Params& P, int d, const double* V) {

@@ -8,6 +8,7 @@
 // and convergence tests stay FP64).  Same launch structure and lanes as rrmhd_f64.cu.
 #include <cuda_runtime.h>
 
+#define RR_DIV_CALLS
 #include "batch.h"
 #include "batch_index.cuh"
 #include "launch_shape.cuh"
@@ -113,7 +114,7 @@ __device__ __forceinline__ int cell_update_f32(const StageArgs& a, int64_t c, co
   const double dt = b.st.dt[q.i];
   float dtdx[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) dtdx[d] = (float)(dt / I.dx[d]);
+  for (int d = 0; d < 3; ++d) dtdx[d] = (float)ddiv(dt, I.dx[d]);
   int64_t fl[3], fr[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -300,8 +301,8 @@ __device__ __forceinline__ void fallback_cell_f32(const StageArgs& a, int64_t c,
     load12(a.Vout, b.ncells, c, Vn);
   }
   if (a.stage == 3 && last) {
-    s = signal_speed(a.P, 0, Vn) / I.dx[0];
-    for (int d = 1; d < I.ndim; ++d) s = s + signal_speed(a.P, d, Vn) / I.dx[d];
+    s = ddiv(signal_speed(a.P, 0, Vn), I.dx[0]);
+    for (int d = 1; d < I.ndim; ++d) s = s + ddiv(signal_speed(a.P, d, Vn), I.dx[d]);
     inst = q.i;
   }
 }

@@ -69,7 +69,7 @@ __device__ __forceinline__ int pvm_flux_tangent(const Params& P, int d, const do
   if (P.beta_mode) {
     double t = tauL > tauR ? tauL : tauR;
     if (t < 1.0) t = 1.0;
-    beta = 1.0 / t;
+    beta = ddiv_call(1.0, t);
   }
   int fail = 1;
   double Vm[NV], Zm = 0.0;
@@ -158,7 +158,7 @@ __device__ __forceinline__ int cell_update(const StageArgs& a, int64_t c, const 
   const double dt = b.st.dt[q.i];
   double dtdx[3];
 #pragma unroll
-  for (int d = 0; d < 3; ++d) dtdx[d] = dt / I.dx[d];
+  for (int d = 0; d < 3; ++d) dtdx[d] = ddiv_call(dt, I.dx[d]);
   int64_t fl[3], fr[3];
 #pragma unroll
   for (int d = 0; d < 3; ++d) {
@@ -362,8 +362,8 @@ __device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, int
     load12(a.Vout, b.ncells, c, Vn);
   }
   if (a.stage == 3 && last) {
-    s = signal_speed(a.P, 0, Vn) / I.dx[0];
-    for (int d = 1; d < I.ndim; ++d) s = s + signal_speed(a.P, d, Vn) / I.dx[d];
+    s = ddiv_call(signal_speed(a.P, 0, Vn), I.dx[0]);
+    for (int d = 1; d < I.ndim; ++d) s = s + ddiv_call(signal_speed(a.P, d, Vn), I.dx[d]);
     inst = q.i;
   }
 }
@@ -465,12 +465,12 @@ __global__ void __launch_bounds__(kFaceThreads) k_bface(StageArgs a) {
   if (has_edges(I, p2)) {
     int q0[3] = {fp.pos[0], fp.pos[1], fp.pos[2]}, q1[3] = {fp.pos[0], fp.pos[1], fp.pos[2]};
     q1[p1] += 1;
-    curl = curl + (a.emf[edge_gidx(b, I, p2, q1)] - a.emf[edge_gidx(b, I, p2, q0)]) / I.dx[p1];
+    curl = curl + ddiv_call(a.emf[edge_gidx(b, I, p2, q1)] - a.emf[edge_gidx(b, I, p2, q0)], I.dx[p1]);
   }
   if (has_edges(I, p1)) {
     int q0[3] = {fp.pos[0], fp.pos[1], fp.pos[2]}, q1[3] = {fp.pos[0], fp.pos[1], fp.pos[2]};
     q1[p2] += 1;
-    curl = curl - (a.emf[edge_gidx(b, I, p1, q1)] - a.emf[edge_gidx(b, I, p1, q0)]) / I.dx[p2];
+    curl = curl - ddiv_call(a.emf[edge_gidx(b, I, p1, q1)] - a.emf[edge_gidx(b, I, p1, q0)], I.dx[p2]);
   }
   double ca = 0.0, cb = 1.0;
   if (a.stage == 2) {
@@ -537,8 +537,8 @@ __global__ void k_signal(Params P, Batch b, const double* __restrict__ V) {
     const InstDesc I = b.inst[i];
     double v[NV];
     load12(V, b.ncells, c, v);
-    s = signal_speed(P, 0, v) / I.dx[0];
-    for (int d = 1; d < I.ndim; ++d) s = s + signal_speed(P, d, v) / I.dx[d];
+    s = ddiv_call(signal_speed(P, 0, v), I.dx[0]);
+    for (int d = 1; d < I.ndim; ++d) s = s + ddiv_call(signal_speed(P, d, v), I.dx[d]);
   }
   warp_smax(b.st.smax, i, (unsigned long long)__double_as_longlong(s));
 }

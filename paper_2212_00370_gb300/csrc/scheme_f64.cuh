@@ -21,7 +21,7 @@ __device__ __forceinline__ double limiter(int recon, double dL, double dR) {
     if (c < m) m = c;
     return dL > 0.0 ? m : -m;
   }
-  return ((2.0 * dL) * dR) / (dL + dR);
+  return ddiv_call((2.0 * dL) * dR, dL + dR);
 }
 
 // Face values of the middle cell: vm at its left face, vp at its right face.
@@ -63,26 +63,6 @@ __device__ __forceinline__ double pvm_alpha(int k, int j) {
   return k == 4 ? PVM16_ALPHA[j] : PVM_ALPHA[j];
 }
 
-// A(U_m)^2 w by two nested flux differences (Sec. 3.2.2 steps 3-5, Eq. utilde).
-// Returns false if a recovery fails.
-__device__ __forceinline__ bool a2_product(const Params& P, int d, const double* Um,
-                                           const double* Fm, double Zm, const double* w,
-                                           double* out) {
-  double Ue[NV], Ve[NV], Fe[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k) Ue[k] = Um[k] + P.pvm_eps * w[k];
-  if (con2prim(P, Ue, Zm, Ve, nullptr) != ST_OK) return false;
-  flux(P, d, Ve, Ue, Fe);
-  // reuse Ue/Ve for U~_eps = U_m + F(U_eps) - F(U_m)
-#pragma unroll
-  for (int k = 0; k < NV; ++k) Ue[k] = Um[k] + (Fe[k] - Fm[k]);
-  if (con2prim(P, Ue, Zm, Ve, nullptr) != ST_OK) return false;
-  flux(P, d, Ve, Ue, Fe);
-#pragma unroll
-  for (int k = 0; k < NV; ++k) out[k] = (Fe[k] - Fm[k]) / P.pvm_eps;
-  return true;
-}
-
 // F^ = (F_L + F_R)/2 - beta p_k(A(U_m)) (U_R - U_L)/2  (Eqs. generalflux, beta),
 // m = 2^(k-1) A^2 products in Horner order (k = 3: PVM-int-8, 4: PVM-int-16);
 // Q = I (lambda_max = 1 Rusanov) if a recovery inside the viscosity term fails.
@@ -90,58 +70,87 @@ __device__ __forceinline__ bool a2_product(const Params& P, int d, const double*
 __device__ __forceinline__ int pvm_flux(const Params& P, int d, const double* VL,
                                         const double* VR, double tauL, double tauR,
                                         double* Fhat) {
-  double Um[NV], U0[NV], Fm[NV], Ul[NV];
-  double ZL, ZR;
+  double Um[NV], U0[NV], Ul[NV];
+  double Zg;
   {
-    double UL[NV], UR[NV], FL[NV], FR[NV];
-    prim2con(P, VL, UL);
-    prim2con(P, VR, UR);
-    flux(P, d, VL, UL, FL);
-    flux(P, d, VR, UR, FR);
+    double Us[NV], Fs[NV];
+    double Z = 0.0;
+#pragma unroll 1
+    for (int side = 0; side < 2; ++side) {
+      const double* V = side ? VR : VL;
+      double U[NV], F[NV];
+      prim2con(P, V, U);
+      flux(P, d, V, U, F);
+      const double Zs = prim_Z(P, V);
+      if (side == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) {
-      U0[k] = UR[k] - UL[k];
-      Um[k] = 0.5 * (UL[k] + UR[k]);
-      Fhat[k] = 0.5 * (FL[k] + FR[k]);  // central part; viscosity subtracted below
+        for (int k = 0; k < NV; ++k) {
+          Us[k] = U[k];
+          Fs[k] = F[k];
+        }
+        Z = Zs;
+      } else {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) {
+          U0[k] = U[k] - Us[k];
+          Um[k] = 0.5 * (Us[k] + U[k]);
+          Fhat[k] = 0.5 * (Fs[k] + F[k]);  // central part; viscosity subtracted below
+        }
+        Zg = 0.5 * (Z + Zs);
+      }
     }
-    ZL = prim_Z(P, VL);
-    ZR = prim_Z(P, VR);
   }
-  const double Zg = 0.5 * (ZL + ZR);
   double beta = 1.0;
   if (P.beta_mode) {
     double t = tauL > tauR ? tauL : tauR;
     if (t < 1.0) t = 1.0;
-    beta = 1.0 / t;
+    beta = ddiv_call(1.0, t);
   }
+  // j = 0: F(U_m).  Then, per A^2 product, two nested flux differences (Sec. 3.2.2 steps
+  // 3-5, Eq. utilde): odd j at U_m + eps U_l, even j at U_m + (F(U_eps) - F(U_m)), whose
+  // flux difference over eps is A^2 U_l.  One loop, one copy of the recovery and the flux.
+  const int m = P.pvm_k == 4 ? 8 : 4;
   int fail = 0;
   double Zm = 0.0;
   {
-    double Vm[NV];
-    if (con2prim(P, Um, Zg, Vm, &Zm) != ST_OK) {
-      fail = 1;
-    } else {
-      flux(P, d, Vm, Um, Fm);
-    }
-  }
-  if (!fail) {
+    double Fm[NV], Y[NV], Ue[NV], Ve[NV], Fe[NV];
+#pragma unroll 1
+    for (int j = 0; j <= 2 * m; ++j) {
+      if (j == 0) {
 #pragma unroll
-    for (int k = 0; k < NV; ++k) Ul[k] = U0[k];
-    const int m = P.pvm_k == 4 ? 8 : 4;
-    for (int l = 0; l < m; ++l) {
-      double Y[NV];
-      if (!a2_product(P, d, Um, Fm, Zm, Ul, Y)) {
+        for (int k = 0; k < NV; ++k) {
+          Ue[k] = Um[k];
+          Ul[k] = U0[k];
+        }
+      } else if (j & 1) {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) Ue[k] = Um[k] + P.pvm_eps * Ul[k];
+      } else {
+#pragma unroll
+        for (int k = 0; k < NV; ++k) Ue[k] = Um[k] + Y[k];
+      }
+      double Z;
+      if (con2prim(P, Ue, j == 0 ? Zg : Zm, Ve, &Z) != ST_OK) {
         fail = 1;
         break;
       }
-      if (l == 0) {
-        const double a0 = pvm_alpha(P.pvm_k, 0), a1 = pvm_alpha(P.pvm_k, 1);
+      flux(P, d, Ve, Ue, Fe);
+      if (j == 0) {
+        Zm = Z;
 #pragma unroll
-        for (int k = 0; k < NV; ++k) Ul[k] = a0 * Y[k] + a1 * U0[k];
+        for (int k = 0; k < NV; ++k) Fm[k] = Fe[k];
       } else {
-        const double al = pvm_alpha(P.pvm_k, l + 1);
 #pragma unroll
-        for (int k = 0; k < NV; ++k) Ul[k] = Y[k] + al * U0[k];
+        for (int k = 0; k < NV; ++k) Y[k] = Fe[k] - Fm[k];
+        if (!(j & 1)) {  // U_l of the next product
+          const int l = j / 2 - 1;
+          const double a0 = pvm_alpha(P.pvm_k, 0), al = pvm_alpha(P.pvm_k, l + 1);
+#pragma unroll
+          for (int k = 0; k < NV; ++k) {
+            const double A2 = ddiv(Y[k], P.pvm_eps);
+            Ul[k] = (l == 0 ? a0 * A2 : A2) + al * U0[k];
+          }
+        }
       }
     }
   }
@@ -169,7 +178,7 @@ __device__ __forceinline__ void hll_block(int k0, int k1, double sL, double sR, 
     else if (sR < 0.0)
       F[k] = FR[k];
     else if (sR > sL)
-      F[k] = ((sR * FL[k] - sL * FR[k]) + (sR * sL) * (UR[k] - UL[k])) / (sR - sL);
+      F[k] = ddiv_call((sR * FL[k] - sL * FR[k]) + (sR * sL) * (UR[k] - UL[k]), sR - sL);
     else
       F[k] = 0.5 * (FL[k] + FR[k]);
   }
@@ -197,7 +206,7 @@ __device__ __forceinline__ void radhll_flux(const Params& P, int d, const double
   double rR = r3L > r3R ? r3L : r3R;
   const double t = tauL > tauR ? tauL : tauR;
   if (P.beta_mode && t > 0.0) {
-    const double lim = 4.0 / (3.0 * t);
+    const double lim = ddiv_call(4.0, 3.0 * t);
     if (rL < -lim) rL = -lim;
     if (rR > lim) rR = lim;
   }
@@ -285,8 +294,8 @@ static __device__ __noinline__ bool imp_residual(const Params& P, const ImpCell&
   } else {
     if (con2prim(P, Um, Zg, V, Z) != ST_OK) return false;
     const double v2 = (V[1] * V[1] + V[2] * V[2]) + V[3] * V[3];
-    W = 1.0 / sqrt(1.0 - v2);
-    T = V[4] / V[0];
+    W = ddiv(1.0, dsqrt(1.0 - v2));
+    T = ddiv(V[4], V[0]);
   }
   const M1 m = m1_coef(X[0], X[1], X[2], X[3]);
   const double u[3] = {W * V[1], W * V[2], W * V[3]};
@@ -328,7 +337,7 @@ __device__ __forceinline__ bool solve4(T A[4][4], T b[4], T x[4]) {
     }
 #pragma unroll
     for (int r = col + 1; r < 4; ++r) {
-      const T f = A[r][col] / A[col][col];
+      const T f = ddiv_call(A[r][col], A[col][col]);
 #pragma unroll
       for (int k = col + 1; k < 4; ++k) A[r][k] = A[r][k] - f * A[col][k];
       b[r] = b[r] - f * b[col];
@@ -339,7 +348,7 @@ __device__ __forceinline__ bool solve4(T A[4][4], T b[4], T x[4]) {
     T s = b[r];
 #pragma unroll
     for (int k = r + 1; k < 4; ++k) s = s - A[r][k] * x[k];
-    x[r] = s / A[r][r];
+    x[r] = ddiv_call(s, A[r][r]);
   }
   return true;
 }
@@ -349,7 +358,7 @@ __device__ __forceinline__ bool solve4(T A[4][4], T b[4], T x[4]) {
 __device__ __forceinline__ void picard_matrix(const ImpCell& c, const double* X,
                                               const double* V, double J[4][4]) {
   const double v2 = (V[1] * V[1] + V[2] * V[2]) + V[3] * V[3];
-  const double W = 1.0 / sqrt(1.0 - v2);
+  const double W = ddiv(1.0, dsqrt(1.0 - v2));
   const double u[3] = {W * V[1], W * V[2], W * V[3]};
   const double rho = V[0];
   double Dr[3][3];
@@ -413,7 +422,7 @@ __device__ __forceinline__ void broyden(JT J[4][4], const double* dXd, const dou
   for (int i = 0; i < 4; ++i) {
     const JT dRi = (JT)(Rn[i] - R[i]);
     const JT Jd = ((J[i][0] * dX[0] + J[i][1] * dX[1]) + J[i][2] * dX[2]) + J[i][3] * dX[3];
-    const JT q = (dRi - Jd) / s2;
+    const JT q = ddiv_call(dRi - Jd, s2);
 #pragma unroll
     for (int j = 0; j < 4; ++j) J[i][j] = J[i][j] + q * dX[j];
   }
@@ -436,7 +445,7 @@ static __device__ __noinline__ bool fd_jacobian(const Params& P, const ImpCell& 
     }
     const double dXj = Xp[j] - X[j];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) J[i][j] = (JT)((Rp[i] - R[i]) / dXj);
+    for (int i = 0; i < 4; ++i) J[i][j] = (JT)(ddiv_call(Rp[i] - R[i], dXj));
   }
   return true;
 }
@@ -546,7 +555,7 @@ static __device__ __noinline__ bool imp_newton(const Params& P, const ImpCell& c
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int j = 0; j < 4; ++j)
-          Mout[4 * i + j] = ((double)J[i][j] - (i == j ? 1.0 : 0.0)) / c.hdt;
+          Mout[4 * i + j] = ddiv_call((double)J[i][j] - (i == j ? 1.0 : 0.0), c.hdt);
       if (F::polish(c, X)) imp_polish<F>(P, c, J, X, R, V, Z, dfull);
       return true;
     }
@@ -610,12 +619,12 @@ static __device__ __noinline__ bool imp_residual_m(const Params& P, const ImpCel
                                                    const double* Y, double* R, double* X,
                                                    double* V) {
   if (!(Y[0] > 0.0)) return false;
-  const double W = sqrt(1.0 + ((Y[1] * Y[1] + Y[2] * Y[2]) + Y[3] * Y[3]));
+  const double W = dsqrt(1.0 + ((Y[1] * Y[1] + Y[2] * Y[2]) + Y[3] * Y[3]));
   double Um[NV];
-  V[0] = c.D / W;
+  V[0] = ddiv_call(c.D, W);
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    V[1 + i] = Y[1 + i] / W;
+    V[1 + i] = ddiv_call(Y[1 + i], W);
     V[5 + i] = c.B[i];
     V[9 + i] = 0.0;
   }
@@ -628,7 +637,7 @@ static __device__ __noinline__ bool imp_residual_m(const Params& P, const ImpCel
   if (!(X[0] > 0.0)) return false;
 #pragma unroll
   for (int i = 0; i < 4; ++i) V[8 + i] = X[i];
-  const double T = Y[0] / V[0];
+  const double T = ddiv_call(Y[0], V[0]);
   const double BP = P.a_rad * ((T * T) * (T * T));
   const M1 m = m1_coef(X[0], X[1], X[2], X[3]);
   double Pr[3][3];
@@ -652,7 +661,7 @@ static __device__ __noinline__ bool imp_newton_m(const Params& P, const ImpCell&
   double R[4];
   if (!imp_residual_m(P, c, Y, R, X, V)) return false;
   for (int m = 1; m <= P.imp_maxit; ++m) {
-    const double su = 1.0 + sqrt((Y[1] * Y[1] + Y[2] * Y[2]) + Y[3] * Y[3]);
+    const double su = 1.0 + dsqrt((Y[1] * Y[1] + Y[2] * Y[2]) + Y[3] * Y[3]);
     const double sc[4] = {Y[0], su, su, su};
     double J[4][4];
     for (int j = 0; j < 4; ++j) {
@@ -665,7 +674,7 @@ static __device__ __noinline__ bool imp_newton_m(const Params& P, const ImpCell&
       }
       const double dYj = Yp[j] - Y[j];
 #pragma unroll
-      for (int i = 0; i < 4; ++i) J[i][j] = (Rp[i] - R[i]) / dYj;
+      for (int i = 0; i < 4; ++i) J[i][j] = ddiv_call(Rp[i] - R[i], dYj);
     }
     double b[4], dY[4];
 #pragma unroll
@@ -723,7 +732,7 @@ static __device__ __noinline__ bool imp_newton_m(const Params& P, const ImpCell&
 __device__ __forceinline__ bool solve_matter(const Params& P, const ImpCell& c, const double* Vs,
                                              double* X, double* V) {
   const double v2 = (Vs[1] * Vs[1] + Vs[2] * Vs[2]) + Vs[3] * Vs[3];
-  const double W = 1.0 / sqrt(1.0 - v2);
+  const double W = ddiv(1.0, dsqrt(1.0 - v2));
   double Y[4] = {Vs[4], W * Vs[1], W * Vs[2], W * Vs[3]};
   return imp_newton_m(P, c, Y, X, V);
 }
@@ -760,7 +769,7 @@ __device__ __forceinline__ int implicit_cell(const Params& P, double kappa, doub
   double X[4] = {c.Xs[0], c.Xs[1], c.Xs[2], c.Xs[3]};
   double R[4], Z = Zguess;
   // no admissible matter state at X*: the explicit update U* itself is inadmissible
-  if constexpr (F::kReuseW) c.iD = 1.0 / c.D;
+  if constexpr (F::kReuseW) c.iD = ddiv_call(1.0, c.D);
   if (!imp_residual<F>(P, c, X, Zguess, R, V, &Z)) return ST_C2P;
   double Mnew[16], Vs[NV];
 #pragma unroll
