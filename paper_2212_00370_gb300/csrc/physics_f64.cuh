@@ -195,15 +195,22 @@ struct C2PPt {  // the root
 // one copy of the evaluation, whatever it is for (the first point, doubled until
 // admissible; Newton points, the step halved until admissible), and f and df are formed
 // only where another Newton step follows.
+// A point is admissible when x > 0 and v^2(x) < 1.  v^2 falls with x (Z = x + D > 0,
+// B^2 >= 0), so every point at or below one whose v^2 came out >= 1 + 1e-9, and every point
+// with Z + B^2 <= |S| (1 - 1e-12), where v^2 >= S^2/(Z + B^2)^2, is inadmissible and is
+// passed over unevaluated: the margins are 10^4 times the rounding of the evaluation.
+// Nearly all halvings are such points (C1, three steps: 35 of 37.7 million, 60 % of all
+// the evaluations of the cell solves).
 // FAST (the FP32-bulk form's cells): 1/Z and 1/(Z+B^2) from one division, W from rsqrt
 // (the same values to a few ulps) and an inexact Newton step with an FP32 reciprocal of
 // df (~6e-8 relative).
 template <bool FAST>
 __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2PPt& e) {
-  double xt = x, dx = 0.0;
+  double xt = x, dx = 0.0, bad = 0.0;
   int it = 0, k = 0;
+  bool bound = false;
   for (;;) {
-    bool ok = xt > 0.0;
+    bool ok = xt > bad;
     double Z, iZ, iZB, iZ2, v2;
     if (ok) {
       Z = xt + c.D;
@@ -219,6 +226,14 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
       iZ2 = iZ * iZ;
       v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * (iZB * iZB);
       ok = v2 < 1.0;
+      if (!ok && c.S2 < 1e200) {
+        if (v2 >= 1.0 + 1e-9) bad = xt;
+        if (!bound) {
+          const double xs = dsqrt_call(c.S2) * (1.0 - 1e-12) - (c.B2 + c.D);
+          if (xs > bad) bad = xs;
+          bound = true;
+        }
+      }
     }
     if (!ok) {
       if (k == (it == 0 ? 200 : 60)) return false;
