@@ -61,6 +61,38 @@ struct Params {
   double gm1g;  // (gamma-1)/gamma
 };
 
+// Products of the pointwise kernels.  SOFT: on the integer pipes (fpi::mul_fast, ~30 integer instructions, 14 clocks
+// per warp and SM against 18.7 on the FP64 pipe, and both pipes run side by side); the
+// factors must be zeros or normal, and the products normal, which the callers' window
+// test ensures.  Same roundings either way.
+template <bool SOFT>
+__device__ __forceinline__ double mul(double a, double b) {
+  if constexpr (SOFT)
+    return fpi::mul_fast<true>(a, b);
+  else
+    return a * b;
+}
+// b + p a for p a power of two: one rounding either way (p a is exact)
+__device__ __forceinline__ double scale_add(double p, double a, double b) {
+#ifdef RR_DIV_CALLS
+  return b + p * a;
+#else
+  return __fma_rn(p, a, b);
+#endif
+}
+
+// Window in which the SOFT products of prim2con and prim_Z are valid: |v| from 2^-200 to 1
+// and |B| within 2^+-100, or zeros; rho and p within 2^+-150.  Every product there has at
+// most six factors and every difference keeps at least the last bit of its terms: all of
+// them stay far inside 2^+-1022 or are exact zeros.
+__device__ __forceinline__ bool soft_matter(const double* V) {
+  using namespace fpi;
+  bool ok = in_window(V[0], 1023 - 150, 300) && in_window(V[4], 1023 - 150, 300);
+#pragma unroll
+  for (int k = 1; k < 4; ++k)
+    ok = ok && in_window_or_zero(V[k], 1023 - 200, 200) && in_window_or_zero(V[4 + k], 1023 - 100, 200);
+  return ok;
+}
 // ---------------------------------------------------------------- aux state
 // W = 1/sqrt(1-v^2), b^0 = W v.B, b^i = B^i/W + v^i b^0, |b|^2 = B^2/W^2 + (v.B)^2,
 // rho h = rho + gamma/(gamma-1) p, p* = p + |b|^2/2   (Sec. 2.1).
@@ -68,45 +100,48 @@ struct Aux {
   double v2, iW, W, vB, B2, b0, b[3], bsq, rhoh, ptot;
 };
 
+template <bool SOFT = false>
 __device__ __forceinline__ void aux_of(const Params& P, const double* V, Aux& a) {
   const double vx = V[1], vy = V[2], vz = V[3];
   const double Bx = V[5], By = V[6], Bz = V[7];
-  a.v2 = (vx * vx + vy * vy) + vz * vz;
+  a.v2 = (mul<SOFT>(vx, vx) + mul<SOFT>(vy, vy)) + mul<SOFT>(vz, vz);
   a.iW = dsqrt(1.0 - a.v2);
   a.W = ddiv(1.0, a.iW);
-  a.vB = (vx * Bx + vy * By) + vz * Bz;
-  a.B2 = (Bx * Bx + By * By) + Bz * Bz;
-  a.b0 = a.W * a.vB;
-  a.b[0] = Bx * a.iW + vx * a.b0;
-  a.b[1] = By * a.iW + vy * a.b0;
-  a.b[2] = Bz * a.iW + vz * a.b0;
-  a.bsq = a.B2 * (a.iW * a.iW) + a.vB * a.vB;
-  a.rhoh = V[0] + P.gfac * V[4];
-  a.ptot = V[4] + 0.5 * a.bsq;
+  a.vB = (mul<SOFT>(vx, Bx) + mul<SOFT>(vy, By)) + mul<SOFT>(vz, Bz);
+  a.B2 = (mul<SOFT>(Bx, Bx) + mul<SOFT>(By, By)) + mul<SOFT>(Bz, Bz);
+  a.b0 = mul<SOFT>(a.W, a.vB);
+  a.b[0] = mul<SOFT>(Bx, a.iW) + mul<SOFT>(vx, a.b0);
+  a.b[1] = mul<SOFT>(By, a.iW) + mul<SOFT>(vy, a.b0);
+  a.b[2] = mul<SOFT>(Bz, a.iW) + mul<SOFT>(vz, a.b0);
+  a.bsq = mul<SOFT>(a.B2, mul<SOFT>(a.iW, a.iW)) + mul<SOFT>(a.vB, a.vB);
+  a.rhoh = V[0] + mul<SOFT>(P.gfac, V[4]);
+  a.ptot = scale_add(0.5, a.bsq, V[4]);
 }
 
 // rho h W^2: the con2prim unknown Z of a primitive state (warm starts).
-__device__ __forceinline__ double prim_Z(const Params& P, const double* V) {
+template <bool SOFT>
+__device__ __forceinline__ double prim_Z_t(const Params& P, const double* V) {
   Aux a;
-  aux_of(P, V, a);
-  return a.rhoh * (a.W * a.W);
+  aux_of<SOFT>(P, V, a);
+  return mul<SOFT>(a.rhoh, mul<SOFT>(a.W, a.W));
 }
 
 // Eq. eqU, with rho W^2 - rho W = D u^2/(W+1) (u^2 = W^2 v^2).
-__device__ __forceinline__ void prim2con(const Params& P, const double* V, double* U) {
+template <bool SOFT>
+__device__ __forceinline__ void prim2con_t(const Params& P, const double* V, double* U) {
   Aux a;
-  aux_of(P, V, a);
-  const double W2 = a.W * a.W;
-  const double D = V[0] * a.W;
-  const double hw = (a.rhoh + a.bsq) * W2;
+  aux_of<SOFT>(P, V, a);
+  const double W2 = mul<SOFT>(a.W, a.W);
+  const double D = mul<SOFT>(V[0], a.W);
+  const double hw = mul<SOFT>(a.rhoh + a.bsq, W2);
   U[0] = D;
-  U[1] = hw * V[1] - a.b0 * a.b[0];
-  U[2] = hw * V[2] - a.b0 * a.b[1];
-  U[3] = hw * V[3] - a.b0 * a.b[2];
-  const double u2 = W2 * a.v2;
-  const double e1 = D * ddiv(u2, a.W + 1.0);
-  const double e2 = (P.gfac * V[4] + a.bsq) * W2;
-  U[4] = (e1 + e2) - (a.ptot + a.b0 * a.b0);
+  U[1] = mul<SOFT>(hw, V[1]) - mul<SOFT>(a.b0, a.b[0]);
+  U[2] = mul<SOFT>(hw, V[2]) - mul<SOFT>(a.b0, a.b[1]);
+  U[3] = mul<SOFT>(hw, V[3]) - mul<SOFT>(a.b0, a.b[2]);
+  const double u2 = mul<SOFT>(W2, a.v2);
+  const double e1 = mul<SOFT>(D, ddiv(u2, a.W + 1.0));
+  const double e2 = mul<SOFT>(mul<SOFT>(P.gfac, V[4]) + a.bsq, W2);
+  U[4] = (e1 + e2) - (a.ptot + mul<SOFT>(a.b0, a.b0));
 #pragma unroll
   for (int k = 5; k < NV; ++k) U[k] = V[k];
 }
@@ -118,7 +153,21 @@ struct M1 {
   double a, c;  // P_ij = c F_i F_j (+ a on the diagonal)
 };
 
+template <bool SOFT = false>
 __device__ __forceinline__ M1 m1_coef(double E, double Fx, double Fy, double Fz) {
+#ifndef RR_DIV_CALLS
+  // factors 2, 4 and 1/2 folded into multiply-adds (their products are exact)
+  const double F2 = (mul<SOFT>(Fx, Fx) + mul<SOFT>(Fy, Fy)) + mul<SOFT>(Fz, Fz);
+  double f2 = ddiv(F2, mul<SOFT>(E, E));
+  if (fpi::gt_nonneg(f2, 1.0)) f2 = 1.0;
+  const double xi = ddiv(__fma_rn(4.0, f2, 3.0), __fma_rn(2.0, dsqrt(4.0 - mul<SOFT>(3.0, f2)), 5.0));
+  M1 m;
+  m.a = mul<SOFT>(__fma_rn(-0.5, xi, 0.5), E);
+  const bool z = !fpi::pos(F2);
+  const double mc = ddiv(mul<SOFT>(__fma_rn(0.5, mul<SOFT>(3.0, xi), -0.5), E), z ? 1.0 : F2);
+  m.c = z ? 0.0 : mc;
+  return m;
+#else
   // uncontracted in every unit: the FP32-bulk unit's results must not depend on how the
   // compiler fuses this sum with what is inlined around it
   const double F2 = __dadd_rn(__dadd_rn(__dmul_rn(Fx, Fx), __dmul_rn(Fy, Fy)), __dmul_rn(Fz, Fz));
@@ -131,10 +180,12 @@ __device__ __forceinline__ M1 m1_coef(double E, double Fx, double Fy, double Fz)
   const double mc = ddiv((0.5 * (3.0 * xi - 1.0)) * E, F2 > 0.0 ? F2 : 1.0);
   if (F2 > 0.0) m.c = mc;
   return m;
+#endif
 }
 
+template <bool SOFT = false>
 __device__ __forceinline__ double m1_P(const M1& m, const double* F, int i, int j) {
-  const double t = m.c * (F[i] * F[j]);
+  const double t = mul<SOFT>(m.c, mul<SOFT>(F[i], F[j]));
   return (i == j) ? t + m.a : t;
 }
 
@@ -180,6 +231,13 @@ __device__ __forceinline__ void flux(const Params& P, int d, const double* V, co
   for (int j = 0; j < 3; ++j) F[9 + j] = m1_P(m, Fr, d, j);
 }
 
+__device__ __forceinline__ double prim_Z(const Params& P, const double* V) {
+  return prim_Z_t<false>(P, V);
+}
+__device__ __forceinline__ void prim2con(const Params& P, const double* V, double* U) {
+  prim2con_t<false>(P, V, U);
+}
+
 // ------------------------------------------------------------- con2prim
 // One-dimensional Newton-Raphson in W' = Z - D, Z = rho h W^2, for the
 // ideal-gas law (Mignone & McKinney 2007); after |dW'| <= 1e-10 W' exactly one
@@ -204,14 +262,43 @@ struct C2PPt {  // the root
 // FAST (the FP32-bulk form's cells): 1/Z and 1/(Z+B^2) from one division, W from rsqrt
 // (the same values to a few ulps) and an inexact Newton step with an FP32 reciprocal of
 // df (~6e-8 relative).
-template <bool FAST>
+// Whether the products of the evaluation may be formed by mul_fast: D and S^2 within
+// 2^+-80, B^2 and (S.B)^2 as well or zero.  With x in [2^-400, 2^80) every factor and every
+// product of the evaluation is then normal (|h| <= 3/Z, the sums that can cancel to zero
+// are tested where they are used).
+__device__ __forceinline__ bool lo_hi_zero(double x) { return fpi::bits(x) == 0; }
+__device__ __forceinline__ bool exp_zero(double x) { return (fpi::hi_word(x) & 0x7ff00000u) == 0; }
+// 0 where z, else x
+__device__ __forceinline__ double zsel(bool z, double x) { return z ? 0.0 : x; }
+__device__ __forceinline__ bool c2p_window(const C2PIn& c) {
+  using namespace fpi;
+  constexpr uint32_t lo = 1023 - 80, n = 160;
+  return in_window(c.D, lo, n) && in_window(c.S2, lo, n) &&
+         (in_window(c.B2, lo, n) || lo_hi_zero(c.B2)) &&
+         (in_window(c.SB2, lo, n) || lo_hi_zero(c.SB2));
+}
+
+// pm: a product of the evaluation inside the window; z: one of its factors is zero.
+template <bool SOFT>
+__device__ __forceinline__ double pm(bool z, double a, double b) {
+  if constexpr (SOFT)
+    return zsel(z, fpi::mul_fast(a, b));
+  else
+    return a * b;
+}
+
+template <bool FAST, bool SOFT>
 __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2PPt& e) {
+  using namespace fpi;
   double xt = x, dx = 0.0, bad = 0.0;
   int it = 0, k = 0;
   bool bound = false;
+  const bool window = !FAST && c2p_window(c);
+  const bool zB = lo_hi_zero(c.B2), zSB = lo_hi_zero(c.SB2);
   for (;;) {
-    bool ok = xt > bad;
-    double Z, iZ, iZB, iZ2, v2;
+    bool ok = gt_nonneg(xt, bad);
+    double Z, iZ, iZB, iZ2, iZB2, v2;
+    const bool in = window && in_window(xt, 1023 - 400, 480);
     if (ok) {
       Z = xt + c.D;
       const double ZB = Z + c.B2;
@@ -219,13 +306,23 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
         const double q = ddiv(1.0, Z * ZB);
         iZ = ZB * q;
         iZB = Z * q;
+        iZ2 = iZ * iZ;
+        v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * (iZB * iZB);
       } else {
         iZ = ddiv(1.0, Z);
         iZB = ddiv(1.0, ZB);
+        if (in) {
+          const double u = __fma_rn(2.0, Z, c.B2);
+          iZ2 = pm<SOFT>(false, iZ, iZ);
+          iZB2 = pm<SOFT>(false, iZB, iZB);
+          v2 = pm<SOFT>(false, c.S2 + pm<SOFT>(zSB, c.SB2, pm<SOFT>(false, u, iZ2)), iZB2);
+        } else {
+          iZ2 = iZ * iZ;
+          iZB2 = iZB * iZB;
+          v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * iZB2;
+        }
       }
-      iZ2 = iZ * iZ;
-      v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * (iZB * iZB);
-      ok = v2 < 1.0;
+      ok = below_one(v2);
       if (!ok && c.S2 < 1e200) {
         if (v2 >= 1.0 + 1e-9) bad = xt;
         if (!bound) {
@@ -248,13 +345,27 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
     }
     x = xt;
     const double omv2 = 1.0 - v2;
-    double W;
-    if constexpr (FAST)
+    double W, p;
+    bool conv;
+    if constexpr (FAST) {
       W = rsqrt(omv2);
-    else
+      p = c.gm1g * (x * omv2 - c.D * ddiv(v2, W + 1.0));
+      conv = mag_le(dx, 1e-10 * x);
+    } else {
       W = ddiv(1.0, dsqrt(omv2));
-    const double p = c.gm1g * (x * omv2 - c.D * ddiv(v2, W + 1.0));
-    if (it > 0 && fabs(dx) <= 1e-10 * x) {
+      const double q = ddiv(v2, W + 1.0);
+      double tol;
+      if (in) {
+        const double t = pm<SOFT>(false, x, omv2) - pm<SOFT>(false, c.D, q);
+        p = pm<SOFT>(exp_zero(t), c.gm1g, t);
+        tol = pm<SOFT>(false, 1e-10, x);
+      } else {
+        p = c.gm1g * (x * omv2 - c.D * q);
+        tol = 1e-10 * x;
+      }
+      conv = mag_le(dx, tol);
+    }
+    if (it > 0 && conv) {
       e.Z = Z;
       e.iZ = iZ;
       e.iZB = iZB;
@@ -264,15 +375,37 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
       return true;
     }
     if (it == maxit) return false;
-    const double f = ((x - p) + (0.5 * c.B2) * (1.0 + v2)) - ((0.5 * c.SB2) * iZ2 + c.tau);
-    const double dv2 = (-2.0 * ((iZB * iZB) * iZB)) *
-                       (c.S2 + c.SB2 * (((3.0 * Z + 3.0 * c.B2) * Z + c.B2 * c.B2) * (iZ2 * iZ)));
-    const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
-    const double df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * (iZ2 * iZ);
     if constexpr (FAST) {
+      const double f = ((x - p) + (0.5 * c.B2) * (1.0 + v2)) - ((0.5 * c.SB2) * iZ2 + c.tau);
+      const double dv2 = (-2.0 * ((iZB * iZB) * iZB)) *
+                         (c.S2 + c.SB2 * (((3.0 * Z + 3.0 * c.B2) * Z + c.B2 * c.B2) * (iZ2 * iZ)));
+      const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
+      const double df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * (iZ2 * iZ);
       const float d32 = (float)df;
       dx = (fabsf(d32) > 1e-30f && fabsf(d32) < 1e30f) ? -f * (double)__frcp_rn(d32) : ddiv(-f, df);
     } else {
+      double f, df;
+      const double opv2 = 1.0 + v2;
+      if (in) {
+        // h = -dv^2/dx / 2.  Factors 2 and 1/2 are folded into multiply-adds (products with
+        // them are exact): the same roundings as with the factor multiplied first.
+        const double fb = __fma_rn(0.5, pm<SOFT>(zB, c.B2, opv2), x - p);
+        f = fb - __fma_rn(0.5, pm<SOFT>(zSB, c.SB2, iZ2), c.tau);
+        const double iZ3 = pm<SOFT>(false, iZ2, iZ), iZB3 = pm<SOFT>(false, iZB2, iZB);
+        const double g = pm<SOFT>(false, pm<SOFT>(false, 3.0, Z) + 3.0 * c.B2, Z) + c.B2 * c.B2;
+        const double h = pm<SOFT>(false, iZB3, c.S2 + pm<SOFT>(zSB, c.SB2, pm<SOFT>(false, g, iZ3)));
+        const double y = __fma_rn(0.5, pm<SOFT>(false, c.D, W), -Z);
+        const double w = __fma_rn(-2.0, pm<SOFT>(exp_zero(y), h, y), omv2);
+        const double dp = pm<SOFT>(exp_zero(w), c.gm1g, w);
+        df = ((1.0 - dp) - pm<SOFT>(zB, c.B2, h)) + pm<SOFT>(zSB, c.SB2, iZ3);
+      } else {
+        f = ((x - p) + (0.5 * c.B2) * opv2) - ((0.5 * c.SB2) * iZ2 + c.tau);
+        const double iZ3 = iZ2 * iZ;
+        const double g = (3.0 * Z + 3.0 * c.B2) * Z + c.B2 * c.B2;
+        const double dv2 = (-2.0 * (iZB2 * iZB)) * (c.S2 + c.SB2 * (g * iZ3));
+        const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
+        df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * iZ3;
+      }
       dx = ddiv(-f, df);
     }
     xt = x + dx;
@@ -287,7 +420,12 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
 // step is taken).  In Newton's quadratic regime the error left is of order
 // (1e-10 x)^2 / x, below rounding, so the PVM's finite-difference products, which
 // differentiate con2prim at the 1e-8 level, see a recovery exact to rounding.
-template <bool FAST = false>
+// SOFT: the products of the evaluation on the integer pipes where the state allows it.  Half
+// of the FP64 instructions less per recovery (1 M C1 states: 825 -> 447 us), but a longer
+// chain (a product is ~100 clocks instead of 64) and 20 KB of code: the faces, whose warps
+// run in step, and the recovery itself take it; the cell solver, paced by its slowest cells
+// and its instruction fetches, does not.
+template <bool FAST = false, bool SOFT = false>
 static __device__ __noinline__ int con2prim(const Params& P, const double* U, double Zguess,
                                             double* V, double* Zout, double* Wout = nullptr) {
   C2PIn c;
@@ -304,12 +442,12 @@ static __device__ __noinline__ int con2prim(const Params& P, const double* U, do
   c.SB = (c.S[0] * c.B[0] + c.S[1] * c.B[1]) + c.S[2] * c.B[2];
   c.SB2 = c.SB * c.SB;
   c.gm1g = P.gm1g;
-  if (!(c.D > 0.0) || !(U[8] > 0.0)) return ST_UNPHYS;
+  if (!fpi::pos(c.D) || !fpi::pos(U[8])) return ST_UNPHYS;
 
   double x = Zguess - c.D;
-  if (!(x > 0.0)) x = (c.tau > 0.0) ? c.tau : c.D;
+  if (!fpi::pos(x)) x = fpi::pos(c.tau) ? c.tau : c.D;
   C2PPt e;
-  if (!c2p_root<FAST>(c, x, P.c2p_maxit, e) || !(e.p > 0.0)) return ST_C2P;
+  if (!c2p_root<FAST, SOFT>(c, x, P.c2p_maxit, e) || !fpi::pos(e.p)) return ST_C2P;
   const double rho = FAST ? c.D * ((1.0 - e.v2) * e.W) : ddiv(c.D, e.W);  // D/W = D (1 - v^2) W
   const double SBiZ = c.SB * e.iZ;
   V[0] = rho;

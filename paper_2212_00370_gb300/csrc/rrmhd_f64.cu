@@ -31,9 +31,12 @@ constexpr int kCellThreads = 128;
 // Resident warps per SM requested from the register allocator for the face and cell
 // kernels (launch-bounds tuning knobs): 0 leaves the registers unbounded (255 per
 // thread, 8 warps per SM); W > 0 asks for W warps per SM in blocks of BS threads (at
-// most 32 resident blocks per SM).
+// most 32 resident blocks per SM).  Faces: with the quotients and the recovery's products
+// on the integer pipes the FP64 pipe is no longer kept busy by 8 warps (flux sweep of
+// 513 x 767: 2.10 ms at 8, 1.90 at 12, 1.96 at 16; 3D box step 90.8, 86.3, 87.2 ms).
+// Cells: 12 and 16 warps are 2-10 % slower, their spills and instruction fetches cost more.
 #ifndef RR_F64_FACE_WARPS
-#define RR_F64_FACE_WARPS 0
+#define RR_F64_FACE_WARPS 12
 #endif
 #ifndef RR_F64_CELL_WARPS
 #define RR_F64_CELL_WARPS 0
@@ -73,7 +76,7 @@ __device__ __forceinline__ int pvm_flux_tangent(const Params& P, int d, const do
   }
   int fail = 1;
   double Vm[NV], Zm = 0.0;
-  if (con2prim(P, Um, Zg, Vm, &Zm) == ST_OK) {
+  if (con2prim<false, true>(P, Um, Zg, Vm, &Zm) == ST_OK) {
     rrt::PT<double> Q;
     Q.gamma = P.gamma;
     Q.gfac = P.gfac;
@@ -618,7 +621,10 @@ __global__ void k_prim2con(Params P, const double* __restrict__ V, double* __res
   if (c >= n) return;
   double v[NV], u[NV];
   load12(V, n, c, v);
-  prim2con(P, v, u);
+  if (soft_matter(v))
+    prim2con_t<true>(P, v, u);
+  else
+    prim2con_t<false>(P, v, u);
 #pragma unroll
   for (int k = 0; k < NV; ++k) U[k * n + c] = u[k];
 }
@@ -640,7 +646,7 @@ __global__ void k_con2prim(Params P, const double* __restrict__ U, const double*
   load12(U, n, c, u);
 #pragma unroll
   for (int k = 0; k < NV; ++k) v[k] = 0.0;
-  const int rc = con2prim(P, u, Zg ? Zg[c] : 0.0, v, nullptr);
+  const int rc = con2prim<false, true>(P, u, Zg ? Zg[c] : 0.0, v, nullptr);
   if (status) status[c] = rc;
 #pragma unroll
   for (int k = 0; k < NV; ++k) V[k * n + c] = v[k];

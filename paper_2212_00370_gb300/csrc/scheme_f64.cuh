@@ -130,7 +130,7 @@ __device__ __forceinline__ int pvm_flux(const Params& P, int d, const double* VL
         for (int k = 0; k < NV; ++k) Ue[k] = Um[k] + Y[k];
       }
       double Z;
-      if (con2prim(P, Ue, j == 0 ? Zg : Zm, Ve, &Z) != ST_OK) {
+      if (con2prim<false, true>(P, Ue, j == 0 ? Zg : Zm, Ve, &Z) != ST_OK) {
         fail = 1;
         break;
       }

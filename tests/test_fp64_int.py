@@ -1,4 +1,4 @@
-"""The integer quotient and square root of fp64_int.cuh are the IEEE ones, bit for bit,
+"""The integer quotient, square root and product of fp64_int.cuh are the IEEE ones, bit for bit,
 whatever the FP32 seed's error within +-2 ulp (host build of the same header)."""
 import os
 import shutil
@@ -66,6 +66,10 @@ int main(int, char** v) {
     const double near[3] = {std::nextafter(p, 0.0), p, std::nextafter(p, 9.0)};
     for (double x : near) check(div_fast<Seed>(x, w), x / w, x, w);
     check(sqrt_fast<Seed>(std::fabs(a)), std::sqrt(std::fabs(a)), a, 0);
+    const double c = from(((1023 + (ea + g() % 400 - 713) / 2) << 52) | mant(g) | (g() & (1ull << 63)));
+    check(mul_fast(c, m), c * m, c, m);                       // and ties: c m with short mantissas
+    check(mul_fast(m, m), m * m, m, m);
+    check(mul_fast<true>(i % 2 ? c : 0.0 * c, i % 3 ? m : -0.0), (i % 2 ? c : 0.0 * c) * (i % 3 ? m : -0.0), c, m);
     const double s = (m + std::ldexp(1.0, -53)) * m;
     check(sqrt_fast<Seed>(s), std::sqrt(s), s, 0);
   }
