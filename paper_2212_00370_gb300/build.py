@@ -31,7 +31,7 @@ UNITS = {
     "rrmhd_server.cu": ["--fmad=false"],
     "rrmhd_probe.cu": [],
 }
-HEADERS = ["fp64_int.cuh", "physics_f64.cuh", "scheme_f64.cuh", "physics_tangent.cuh", "batch.h", "batch_index.cuh",
+HEADERS = ["fp64_int.cuh", "physics_f64.cuh", "scheme_f64.cuh", "implicit_warp.cuh", "physics_tangent.cuh", "batch.h", "batch_index.cuh",
            "engine.h", "launch_shape.cuh"]
 
 

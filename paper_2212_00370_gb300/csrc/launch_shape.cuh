@@ -39,6 +39,34 @@ __device__ __forceinline__ void persistent_items(int64_t n, unsigned long long* 
   }
 }
 
+// The same schedules for items that a warp works on together: f(t, have, mask) is called by
+// every thread of a warp that has an item at all (have: this thread's t is one; mask: the
+// warp's threads).
+template <int BS, int PT, class F>
+__device__ __forceinline__ void grid_items_warp(int64_t n, F&& f) {
+  constexpr unsigned mask = BS < 32 ? (1u << (BS & 31)) - 1u : 0xffffffffu;
+  const int64_t base = (int64_t)blockIdx.x * (BS * PT) + threadIdx.x;
+#pragma unroll
+  for (int j = 0; j < PT; ++j) {
+    const int64_t t = base + (int64_t)j * BS;
+    if (t - (int64_t)(threadIdx.x & 31) < n) f(t, t < n, mask);
+  }
+}
+
+template <class F>
+__device__ __forceinline__ void persistent_items_warp(int64_t n, unsigned long long* counter, F&& f) {
+  const int lane = threadIdx.x & 31;
+  while (true) {
+    unsigned long long base = 0;
+    __syncwarp();
+    if (lane == 0) base = atomicAdd(counter, 32ull);
+    base = __shfl_sync(0xffffffffu, base, 0);
+    if (base >= (unsigned long long)n) break;
+    const int64_t t = (int64_t)base + lane;
+    f(t, t < n);
+  }
+}
+
 // The shapes that are compiled: block size x items per thread (grid schedule) and
 // block size (persistent schedule).
 // Blocks of 8 and 16 threads (grid schedule, one item per thread) spread a small

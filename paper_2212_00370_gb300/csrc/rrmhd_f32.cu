@@ -13,7 +13,7 @@
 #include "batch_index.cuh"
 #include "launch_shape.cuh"
 #include "physics_tangent.cuh"
-#include "scheme_f64.cuh"
+#include "implicit_warp.cuh"
 
 namespace rr {
 
@@ -107,8 +107,8 @@ static __device__ __noinline__ void face_item_f32(const StageArgs& a, int64_t t)
 }
 
 // U* with the flux difference in FP32, accumulated into FP64; FP64 implicit solve.
-__device__ __forceinline__ int cell_update_f32(const StageArgs& a, int64_t c, const CellPos& q,
-                                               double* Un, double* Vn) {
+__device__ __forceinline__ void cell_begin_f32(const StageArgs& a, int64_t c, const CellPos& q,
+                                               ImpTask<FormBulk>& t, double* Ust) {
   const Batch& b = a.b;
   const InstDesc& I = q.I;
   const double dt = b.st.dt[q.i];
@@ -138,7 +138,6 @@ __device__ __forceinline__ int cell_update_f32(const StageArgs& a, int64_t c, co
   }
   const int64_t N = b.ncells;
   const int64_t FS = a.fstride;
-  double Ust[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     float acc = (a.Fhat32[k * FS + fr[0]] - a.Fhat32[k * FS + fl[0]]) * dtdx[0];
@@ -153,10 +152,7 @@ __device__ __forceinline__ int cell_update_f32(const StageArgs& a, int64_t c, co
   double jc[17];
 #pragma unroll
   for (int k = 0; k < 17; ++k) jc[k] = a.jc[k * N + c];
-  const int rc = implicit_cell<FormBulk>(a.P, a.kappa[c], a.sigma[c], cw * dt, Ust, prim_Z(a.P, vs), Un, Vn, jc);
-#pragma unroll
-  for (int k = 0; k < 17; ++k) a.jc[k * N + c] = jc[k];
-  return rc;
+  imp_begin(a.P, t, a.kappa[c], a.sigma[c], cw * dt, Ust, prim_Z(a.P, vs), jc);
 }
 
 __device__ __forceinline__ void store_cell(const StageArgs& a, int64_t c, const double* Un,
@@ -169,12 +165,38 @@ __device__ __forceinline__ void store_cell(const StageArgs& a, int64_t c, const 
   }
 }
 
-static __device__ __noinline__ void cell_item_f32(const StageArgs& a, int64_t c) {
-  const CellPos q = cell_pos(a.b, c);
-  if (!inst_active(a.b, q.i)) return;
-  double Un[NV], Vn[NV];
-  const int rc = cell_update_f32(a, c, q, Un, Vn);
-  if (a.cell_status) a.cell_status[c] = rc;
+// The cell's solve is done: its cache, and on success its state.  Returns the Status.
+__device__ __forceinline__ int cell_end_f32(const StageArgs& a, int64_t c, const ImpTask<FormBulk>& t,
+                                        const double* Ust) {
+  const int64_t N = a.b.ncells;
+#pragma unroll
+  for (int k = 0; k < 17; ++k) a.jc[k * N + c] = t.jc[k];
+  if (a.cell_status) a.cell_status[c] = t.rc;
+  if (t.rc == ST_OK) {
+    double Un[NV];
+    imp_result(t, Ust, Un);
+    store_cell(a, c, Un, t.V);
+  }
+  return t.rc;
+}
+
+// Pass 1: every cell.  A cell whose U* is inadmissible is only flagged.  Every lane of the
+// warp (mask) calls it; have: the lane has a cell.
+static __device__ __noinline__ void cell_item_f32(const StageArgs& a, int64_t c, bool have,
+                                              unsigned mask) {
+  ImpTask<FormBulk> t;
+  t.phase = IMP_DONE;
+  double Ust[NV];
+  int inst = 0;
+  if (have) {
+    const CellPos q = cell_pos(a.b, c);
+    inst = q.i;
+    have = inst_active(a.b, q.i);
+    if (have) cell_begin_f32(a, c, q, t, Ust);
+  }
+  implicit_warp(a.P, mask, t);
+  if (!have) return;
+  const int rc = cell_end_f32(a, c, t, Ust);
   const bool retry = fallback_retry(rc);
   a.bad[c] = retry ? 1 : 0;
   if (retry) {
@@ -182,11 +204,9 @@ static __device__ __noinline__ void cell_item_f32(const StageArgs& a, int64_t c)
     return;
   }
   if (rc != ST_OK) {
-    atomicCAS(a.b.st.status + q.i, 0, rc);
-    if (a.b.st.bad_cell) atomicMin(a.b.st.bad_cell + q.i, (long long)c);
-    return;
+    atomicCAS(a.b.st.status + inst, 0, rc);
+    if (a.b.st.bad_cell) atomicMin(a.b.st.bad_cell + inst, (long long)c);
   }
-  store_cell(a, c, Un, Vn);
 }
 
 template <int BS, int PT>
@@ -201,13 +221,16 @@ __global__ void __launch_bounds__(BS, RR_F32_FACE_BLOCKS(BS)) k_faces_f32_persis
 
 template <int BS, int PT>
 __global__ void __launch_bounds__(BS, RR_F32_CELL_BLOCKS(BS)) k_cells_f32(StageArgs a) {
-  grid_items<BS, PT>(a.b.c_end - a.b.c_begin, [&](int64_t t) { cell_item_f32(a, a.b.c_begin + t); });
+  grid_items_warp<BS, PT>(a.b.c_end - a.b.c_begin, [&](int64_t t, bool have, unsigned mask) {
+    cell_item_f32(a, a.b.c_begin + t, have, mask);
+  });
 }
 
 template <int BS>
 __global__ void __launch_bounds__(BS, RR_F32_CELL_BLOCKS(BS)) k_cells_f32_persistent(StageArgs a) {
-  persistent_items(a.b.c_end - a.b.c_begin, a.work + 1,
-                   [&](int64_t t) { cell_item_f32(a, a.b.c_begin + t); });
+  persistent_items_warp(a.b.c_end - a.b.c_begin, a.work + 1, [&](int64_t t, bool have) {
+    cell_item_f32(a, a.b.c_begin + t, have, 0xffffffffu);
+  });
 }
 
 __global__ void __launch_bounds__(kFaceThreads) k_fallback_faces_f32(StageArgs a) {
@@ -236,26 +259,28 @@ __global__ void __launch_bounds__(kFaceThreads) k_fallback_faces_f32(StageArgs a
 
 // One cell of a fallback pass; in the last pass of stage 3, inst and s receive the
 // cell's instance and CFL signal speed (left at -1 where the cell adds none).
-__device__ __forceinline__ void fallback_cell_f32(const StageArgs& a, int64_t c, int& inst,
-                                                  double& s) {
+__device__ __forceinline__ void fallback_cell_f32(const StageArgs& a, int64_t c, bool have, int& inst,
+                                              double& s) {
   const Batch& b = a.b;
-  const CellPos q = cell_pos(b, c);
   const int pass = a.fb_pass;
   const bool last = pass == kFallbackPasses;
   const bool none = a.flagged && a.flagged[pass] == 0;  // no cell flagged in this pass
+  // (the same on every lane: the warp returns together)
   if (none && !(a.stage == 3 && last)) return;
-  if (!inst_active(b, q.i)) {
+  CellPos q;
+  if (have) q = cell_pos(b, c);
+  if (have && !inst_active(b, q.i)) {
     if (a.stage == 3 && last) {
       double u[NV], v[NV];
       load12(a.U0, b.ncells, c, u);
       load12(a.V0, b.ncells, c, v);
       store_cell(a, c, u, v);
     }
-    return;
+    have = false;
   }
   const InstDesc& I = q.I;
-  bool hit = !none && a.bad[c] == pass;
-  if (!none && !hit && a.ct && I.ndim >= 2) {
+  bool hit = have && !none && a.bad[c] == pass;
+  if (have && !none && !hit && a.ct && I.ndim >= 2) {
     // constrained transport: the face field changes on every face that meets a
     // flagged cell's edges, so the whole 3x3(x3) block around it is updated again
     const int lo2 = I.ndim == 3 ? -1 : 0, hi2 = I.ndim == 3 ? 1 : 0;
@@ -272,7 +297,7 @@ __device__ __forceinline__ void fallback_cell_f32(const StageArgs& a, int64_t c,
           if (in && a.bad[I.cell_off + ((int64_t)r[2] * I.n[1] + r[1]) * I.n[0] + r[0]] == pass) hit = true;
         }
   }
-  for (int d = 0; d < I.ndim && !hit && !none; ++d) {
+  for (int d = 0; have && d < I.ndim && !hit && !none; ++d) {
     for (int e = -1; e <= 1; e += 2) {
       const int pd = q.p[d] + e;
       if ((pd < 0 || pd >= I.n[d]) && I.bc[d] != 1) continue;
@@ -281,11 +306,14 @@ __device__ __forceinline__ void fallback_cell_f32(const StageArgs& a, int64_t c,
       if (a.bad[I.cell_off + ((int64_t)r[2] * I.n[1] + r[1]) * I.n[0] + r[0]] == pass) hit = true;
     }
   }
-  double Vn[NV];
+  ImpTask<FormBulk> t;
+  t.phase = IMP_DONE;
+  double Ust[NV];
+  if (hit) cell_begin_f32(a, c, q, t, Ust);
+  if (!none) implicit_warp(a.P, 0xffffffffu, t);
+  if (!have) return;
   if (hit) {
-    double Un[NV];
-    const int rc = cell_update_f32(a, c, q, Un, Vn);
-    if (a.cell_status) a.cell_status[c] = rc;
+    const int rc = cell_end_f32(a, c, t, Ust);
     if (fallback_retry(rc) && a.bad[c] == 0 && !last) {
       a.bad[c] = (uint8_t)(pass + 1);  // its faces go first-order in the next pass
       if (a.flagged) atomicAdd(a.flagged + pass + 1, 1u);
@@ -296,13 +324,12 @@ __device__ __forceinline__ void fallback_cell_f32(const StageArgs& a, int64_t c,
       if (b.st.bad_cell) atomicMin(b.st.bad_cell + q.i, (long long)c);
       return;
     }
-    store_cell(a, c, Un, Vn);
   } else if (a.stage == 3 && last) {
-    load12(a.Vout, b.ncells, c, Vn);
+    load12(a.Vout, b.ncells, c, t.V);
   }
   if (a.stage == 3 && last) {
-    s = ddiv(signal_speed(a.P, 0, Vn), I.dx[0]);
-    for (int d = 1; d < I.ndim; ++d) s = s + ddiv(signal_speed(a.P, d, Vn), I.dx[d]);
+    s = ddiv(signal_speed(a.P, 0, t.V), I.dx[0]);
+    for (int d = 1; d < I.ndim; ++d) s = s + ddiv(signal_speed(a.P, d, t.V), I.dx[d]);
     inst = q.i;
   }
 }
@@ -311,7 +338,7 @@ __global__ void __launch_bounds__(kCellThreads) k_fallback_cells_f32(StageArgs a
   const int64_t c = a.b.c_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int inst = -1;
   double s = 0.0;
-  if (c < a.b.c_end) fallback_cell_f32(a, c, inst, s);
+  fallback_cell_f32(a, c, c < a.b.c_end, inst, s);
   // the CFL maximum of the next step (launch-uniform condition: every lane gets here)
   if (a.stage == 3 && a.fb_pass == kFallbackPasses)
     warp_smax(a.b.st.smax, inst, (unsigned long long)__double_as_longlong(s));

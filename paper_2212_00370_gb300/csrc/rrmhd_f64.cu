@@ -19,7 +19,7 @@
 #include "batch_index.cuh"
 #include "launch_shape.cuh"
 #include "physics_tangent.cuh"
-#include "scheme_f64.cuh"
+#include "implicit_warp.cuh"
 
 namespace rr {
 
@@ -154,8 +154,8 @@ static __device__ __noinline__ void face_item(const StageArgs& a, int64_t t) {
 
 // U* of cell c from its face fluxes (flux difference and RK combination,
 // Sec. 3.1), then the implicit solve (Sec. 3.3); returns a Status.
-__device__ __forceinline__ int cell_update(const StageArgs& a, int64_t c, const CellPos& q,
-                                           double* Un, double* Vn) {
+__device__ __forceinline__ void cell_begin(const StageArgs& a, int64_t c, const CellPos& q,
+                                           ImpTask<FormF64>& t, double* Ust) {
   const Batch& b = a.b;
   const InstDesc& I = q.I;
   const double dt = b.st.dt[q.i];
@@ -186,7 +186,6 @@ __device__ __forceinline__ int cell_update(const StageArgs& a, int64_t c, const 
   const double hdt = cw * dt;
   const int64_t N = b.ncells;
   const int64_t FS = a.fstride;
-  double Ust[NV];
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     double acc = (a.Fhat[k * FS + fr[0]] - a.Fhat[k * FS + fl[0]]) * dtdx[0];
@@ -206,10 +205,7 @@ __device__ __forceinline__ int cell_update(const StageArgs& a, int64_t c, const 
   double jc[17];
 #pragma unroll
   for (int k = 0; k < 17; ++k) jc[k] = a.jc[k * N + c];
-  const int rc = implicit_cell(a.P, a.kappa[c], a.sigma[c], hdt, Ust, Zg, Un, Vn, jc);
-#pragma unroll
-  for (int k = 0; k < 17; ++k) a.jc[k * N + c] = jc[k];
-  return rc;
+  imp_begin(a.P, t, a.kappa[c], a.sigma[c], hdt, Ust, Zg, jc);
 }
 
 __device__ __forceinline__ void store_cell(const StageArgs& a, int64_t c, const double* Un,
@@ -222,13 +218,38 @@ __device__ __forceinline__ void store_cell(const StageArgs& a, int64_t c, const 
   }
 }
 
-// Pass 1: every cell.  A cell whose U* is inadmissible is only flagged.
-static __device__ __noinline__ void cell_item(const StageArgs& a, int64_t c) {
-  const CellPos q = cell_pos(a.b, c);
-  if (!inst_active(a.b, q.i)) return;
-  double Un[NV], Vn[NV];
-  const int rc = cell_update(a, c, q, Un, Vn);
-  if (a.cell_status) a.cell_status[c] = rc;
+// The cell's solve is done: its cache, and on success its state.  Returns the Status.
+__device__ __forceinline__ int cell_end(const StageArgs& a, int64_t c, const ImpTask<FormF64>& t,
+                                        const double* Ust) {
+  const int64_t N = a.b.ncells;
+#pragma unroll
+  for (int k = 0; k < 17; ++k) a.jc[k * N + c] = t.jc[k];
+  if (a.cell_status) a.cell_status[c] = t.rc;
+  if (t.rc == ST_OK) {
+    double Un[NV];
+    imp_result(t, Ust, Un);
+    store_cell(a, c, Un, t.V);
+  }
+  return t.rc;
+}
+
+// Pass 1: every cell.  A cell whose U* is inadmissible is only flagged.  Every lane of the
+// warp (mask) calls it; have: the lane has a cell.
+static __device__ __noinline__ void cell_item(const StageArgs& a, int64_t c, bool have,
+                                              unsigned mask) {
+  ImpTask<FormF64> t;
+  t.phase = IMP_DONE;
+  double Ust[NV];
+  int inst = 0;
+  if (have) {
+    const CellPos q = cell_pos(a.b, c);
+    inst = q.i;
+    have = inst_active(a.b, q.i);
+    if (have) cell_begin(a, c, q, t, Ust);
+  }
+  implicit_warp(a.P, mask, t);
+  if (!have) return;
+  const int rc = cell_end(a, c, t, Ust);
   const bool retry = fallback_retry(rc);
   a.bad[c] = retry ? 1 : 0;
   if (retry) {
@@ -236,11 +257,9 @@ static __device__ __noinline__ void cell_item(const StageArgs& a, int64_t c) {
     return;
   }
   if (rc != ST_OK) {
-    atomicCAS(a.b.st.status + q.i, 0, rc);
-    if (a.b.st.bad_cell) atomicMin(a.b.st.bad_cell + q.i, (long long)c);
-    return;
+    atomicCAS(a.b.st.status + inst, 0, rc);
+    if (a.b.st.bad_cell) atomicMin(a.b.st.bad_cell + inst, (long long)c);
   }
-  store_cell(a, c, Un, Vn);
 }
 
 template <int BS, int PT>
@@ -255,13 +274,16 @@ __global__ void __launch_bounds__(BS, RR_F64_BLOCKS(RR_F64_FACE_WARPS, BS)) k_fa
 
 template <int BS, int PT>
 __global__ void __launch_bounds__(BS, RR_F64_BLOCKS(RR_F64_CELL_WARPS, BS)) k_cells(StageArgs a) {
-  grid_items<BS, PT>(a.b.c_end - a.b.c_begin, [&](int64_t t) { cell_item(a, a.b.c_begin + t); });
+  grid_items_warp<BS, PT>(a.b.c_end - a.b.c_begin, [&](int64_t t, bool have, unsigned mask) {
+    cell_item(a, a.b.c_begin + t, have, mask);
+  });
 }
 
 template <int BS>
 __global__ void __launch_bounds__(BS, RR_F64_BLOCKS(RR_F64_CELL_WARPS, BS)) k_cells_persistent(StageArgs a) {
-  persistent_items(a.b.c_end - a.b.c_begin, a.work + 1,
-                   [&](int64_t t) { cell_item(a, a.b.c_begin + t); });
+  persistent_items_warp(a.b.c_end - a.b.c_begin, a.work + 1, [&](int64_t t, bool have) {
+    cell_item(a, a.b.c_begin + t, have, 0xffffffffu);
+  });
 }
 
 // Admissibility fallback, pass a.fb_pass, faces: first-order Rusanov flux at
@@ -299,14 +321,17 @@ __global__ void __launch_bounds__(kFaceThreads) k_fallback_faces(StageArgs a) {
 // inactive instances over.
 // One cell of a fallback pass; in the last pass of stage 3, inst and s receive the
 // cell's instance and CFL signal speed (left at -1 where the cell adds none).
-__device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, int& inst, double& s) {
+__device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, bool have, int& inst,
+                                              double& s) {
   const Batch& b = a.b;
-  const CellPos q = cell_pos(b, c);
   const int pass = a.fb_pass;
   const bool last = pass == kFallbackPasses;
   const bool none = a.flagged && a.flagged[pass] == 0;  // no cell flagged in this pass
+  // (the same on every lane: the warp returns together)
   if (none && !(a.stage == 3 && last)) return;
-  if (!inst_active(b, q.i)) {
+  CellPos q;
+  if (have) q = cell_pos(b, c);
+  if (have && !inst_active(b, q.i)) {
     // finished or failed instance: carry its start-of-step state into the
     // step's output buffers (a failed instance stays at its last good state)
     if (a.stage == 3 && last) {
@@ -315,11 +340,11 @@ __device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, int
       load12(a.V0, b.ncells, c, v);
       store_cell(a, c, u, v);
     }
-    return;
+    have = false;
   }
   const InstDesc& I = q.I;
-  bool hit = !none && a.bad[c] == pass;
-  if (!none && !hit && a.ct && I.ndim >= 2) {
+  bool hit = have && !none && a.bad[c] == pass;
+  if (have && !none && !hit && a.ct && I.ndim >= 2) {
     // constrained transport: the face field changes on every face that meets a
     // flagged cell's edges, so the whole 3x3(x3) block around it is updated again
     const int lo2 = I.ndim == 3 ? -1 : 0, hi2 = I.ndim == 3 ? 1 : 0;
@@ -336,7 +361,7 @@ __device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, int
           if (in && a.bad[I.cell_off + ((int64_t)r[2] * I.n[1] + r[1]) * I.n[0] + r[0]] == pass) hit = true;
         }
   }
-  for (int d = 0; d < I.ndim && !hit && !none; ++d) {
+  for (int d = 0; have && d < I.ndim && !hit && !none; ++d) {
     for (int e = -1; e <= 1; e += 2) {
       const int pd = q.p[d] + e;
       if ((pd < 0 || pd >= I.n[d]) && I.bc[d] != 1) continue;  // outflow ghost face
@@ -345,11 +370,14 @@ __device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, int
       if (a.bad[I.cell_off + ((int64_t)r[2] * I.n[1] + r[1]) * I.n[0] + r[0]] == pass) hit = true;
     }
   }
-  double Vn[NV];
+  ImpTask<FormF64> t;
+  t.phase = IMP_DONE;
+  double Ust[NV];
+  if (hit) cell_begin(a, c, q, t, Ust);
+  if (!none) implicit_warp(a.P, 0xffffffffu, t);
+  if (!have) return;
   if (hit) {
-    double Un[NV];
-    const int rc = cell_update(a, c, q, Un, Vn);
-    if (a.cell_status) a.cell_status[c] = rc;
+    const int rc = cell_end(a, c, t, Ust);
     if (fallback_retry(rc) && a.bad[c] == 0 && !last) {
       a.bad[c] = (uint8_t)(pass + 1);  // its faces go first-order in the next pass
       if (a.flagged) atomicAdd(a.flagged + pass + 1, 1u);
@@ -360,13 +388,12 @@ __device__ __forceinline__ void fallback_cell(const StageArgs& a, int64_t c, int
       if (b.st.bad_cell) atomicMin(b.st.bad_cell + q.i, (long long)c);
       return;
     }
-    store_cell(a, c, Un, Vn);
   } else if (a.stage == 3 && last) {
-    load12(a.Vout, b.ncells, c, Vn);
+    load12(a.Vout, b.ncells, c, t.V);
   }
   if (a.stage == 3 && last) {
-    s = ddiv_call(signal_speed(a.P, 0, Vn), I.dx[0]);
-    for (int d = 1; d < I.ndim; ++d) s = s + ddiv_call(signal_speed(a.P, d, Vn), I.dx[d]);
+    s = ddiv_call(signal_speed(a.P, 0, t.V), I.dx[0]);
+    for (int d = 1; d < I.ndim; ++d) s = s + ddiv_call(signal_speed(a.P, d, t.V), I.dx[d]);
     inst = q.i;
   }
 }
@@ -375,7 +402,7 @@ __global__ void __launch_bounds__(kCellThreads, RR_F64_BLOCKS(RR_F64_CELL_WARPS,
   const int64_t c = a.b.c_begin + (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int inst = -1;
   double s = 0.0;
-  if (c < a.b.c_end) fallback_cell(a, c, inst, s);
+  fallback_cell(a, c, c < a.b.c_end, inst, s);
   // the CFL maximum of the next step (launch-uniform condition: every lane gets here)
   if (a.stage == 3 && a.fb_pass == kFallbackPasses)
     warp_smax(a.b.st.smax, inst, (unsigned long long)__double_as_longlong(s));
@@ -652,26 +679,31 @@ __global__ void k_con2prim(Params P, const double* __restrict__ U, const double*
   for (int k = 0; k < NV; ++k) V[k * n + c] = v[k];
 }
 
-__global__ void k_implicit(Params P, Batch b, double hdt, const double* __restrict__ Us,
-                           const double* __restrict__ Zg, const double* __restrict__ kappa,
-                           const double* __restrict__ sigma, double* __restrict__ U,
-                           double* __restrict__ V, int32_t* __restrict__ status) {
+__global__ void __launch_bounds__(kCellThreads) k_implicit(
+    Params P, Batch b, double hdt, const double* __restrict__ Us, const double* __restrict__ Zg,
+    const double* __restrict__ kappa, const double* __restrict__ sigma, double* __restrict__ U,
+    double* __restrict__ V, int32_t* __restrict__ status) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = b.ncells;
-  if (c >= n) return;
-  double us[NV], un[NV], vn[NV];
-  load12(Us, n, c, us);
+  ImpTask<FormF64> t;
+  t.phase = IMP_DONE;
+  double us[NV], un[NV];
+  if (c < n) {
+    load12(Us, n, c, us);
 #pragma unroll
-  for (int k = 0; k < NV; ++k) {
-    un[k] = 0.0;
-    vn[k] = 0.0;
+    for (int k = 0; k < NV; ++k) t.V[k] = 0.0;
+    imp_begin(P, t, kappa[c], sigma[c], hdt, us, Zg ? Zg[c] : 0.0, nullptr);
   }
-  const int rc = implicit_cell(P, kappa[c], sigma[c], hdt, us, Zg ? Zg[c] : 0.0, un, vn);
-  if (status) status[c] = rc;
+  implicit_warp(P, 0xffffffffu, t);
+  if (c >= n) return;
+#pragma unroll
+  for (int k = 0; k < NV; ++k) un[k] = 0.0;
+  if (t.rc == ST_OK || t.m == 0) imp_result(t, us, un);
+  if (status) status[c] = t.rc;
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
     U[k * n + c] = un[k];
-    V[k * n + c] = vn[k];
+    V[k * n + c] = t.V[k];
   }
 }
 

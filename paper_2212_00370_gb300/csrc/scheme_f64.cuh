@@ -428,186 +428,10 @@ __device__ __forceinline__ void broyden(JT J[4][4], const double* dXd, const dou
   }
 }
 
-// Forward-difference Jacobian of R at X (step 1e-7 E_r; a backward step where the
-// forward one leaves the admissible set).  False if neither is admissible.
-template <class F>
-static __device__ __noinline__ bool fd_jacobian(const Params& P, const ImpCell& c, const double* X,
-                                                const double* R, double Z, typename F::Mat J[4][4]) {
-  using JT = typename F::Mat;
-  const double h = 1e-7 * X[0];
-  for (int j = 0; j < 4; ++j) {
-    double Xp[4] = {X[0], X[1], X[2], X[3]};
-    double Rp[4], Vp[NV], Zp;
-    Xp[j] = X[j] + h;
-    if (!imp_residual<F>(P, c, Xp, Z, Rp, Vp, &Zp)) {
-      Xp[j] = X[j] - h;
-      if (!imp_residual<F>(P, c, Xp, Z, Rp, Vp, &Zp)) return false;
-    }
-    const double dXj = Xp[j] - X[j];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) J[i][j] = (JT)(ddiv_call(Rp[i] - R[i], dXj));
-  }
-  return true;
-}
-
 constexpr double IMP_POLISH_TOL = 1e-14;  // polished root: last correction <= 1e-14 E_r
 constexpr int IMP_POLISH_MAX = 6;         // at most six polishing corrections
 
-// Polish of a converged iterate.  Stopping at imp_tol leaves an error of about the
-// last step times the matrix's contraction, which depends on how the iterate was
-// reached (first matrix, Broyden history, the cell's cache).  The iterate is refined
-// towards the root of R itself, so that the result is a function of the cell's state:
-// corrections dX = -J^-1 R(X), accepted without line search, J updated by Broyden's
-// formula after each, until a correction is <= 1e-14 E_r.  A correction that does not
-// halve the previous one means the rounding floor of R is reached: the polish stops
-// there without taking it.  last is the size of the converged step.  X, R, V and Z
-// stay those of the last accepted iterate.
-template <class F>
-static __device__ __noinline__ void imp_polish(const Params& P, const ImpCell& c, typename F::Mat J[4][4],
-                                               double* X, double* R, double* V, double* Z,
-                                               double last) {
-  double prev = last;
-  for (int p = 0; p < IMP_POLISH_MAX; ++p) {
-    double dX[4];
-    if (!newton_dir(J, R, dX)) return;
-    double d = 0.0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) d = fabs(dX[i]) > d ? fabs(dX[i]) : d;
-    if (d <= IMP_POLISH_TOL * X[0]) return;
-    if (p > 0 && d > 0.5 * prev) return;
-    double Xn[4], Rn[4], Vn[NV], Zn = *Z;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) Xn[i] = X[i] + dX[i];
-    if (!imp_residual<F>(P, c, Xn, *Z, Rn, Vn, &Zn)) return;
-    broyden(J, dX, R, Rn);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      X[i] = Xn[i];
-      R[i] = Rn[i];
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) V[k] = Vn[k];
-    *Z = Zn;
-    prev = d;
-  }
-}
-
-// Quasi-Newton iteration on R(X) = 0: first matrix C^(m) (the paper's
-// frozen-matter iteration), Broyden rank-one update after every accepted step,
-// forward-difference Jacobian (step 1e-7 E_r) when successive steps contract by
-// less than 2x or no descent is found; Armijo backtracking on |R|^2 (at most ten
-// halvings); converged
-// when the full step is <= imp_tol * E_r, then polished (imp_polish).  Returns true
-// on convergence.
-template <class F>
-static __device__ __noinline__ bool imp_newton(const Params& P, const ImpCell& c, double* X, double* R,
-                                               double* V, double* Z, const double* Min, double* Mout) {
-  using JT = typename F::Mat;
-  JT J[4][4];
-  int need_fd = 0, fresh_fd = 0, first = 1;
-  double prev = -1.0;
-  if (Min) {  // the cell's matrix from its previous solve: J = I + h M
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) J[i][j] = (JT)((i == j ? 1.0 : 0.0) + c.hdt * Min[4 * i + j]);
-  } else {
-    double Jd[4][4];
-    picard_matrix(c, X, V, Jd);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) J[i][j] = (JT)Jd[i][j];
-  }
-  for (int m = 1; m <= P.imp_maxit; ++m) {
-    if (need_fd) {
-      if (!fd_jacobian<F>(P, c, X, R, *Z, J)) return false;
-      need_fd = 0;
-      fresh_fd = 1;
-      first = 0;
-    }
-    double dX[4];
-    if (!newton_dir(J, R, dX)) {
-      if (!fresh_fd) {
-        need_fd = 1;
-        continue;
-      }
-      return false;
-    }
-
-    double dfull = 0.0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) dfull = fabs(dX[i]) > dfull ? fabs(dX[i]) : dfull;
-    double Xn[4], Rn[4], Vn[NV], Zn = *Z;
-    if (dfull <= P.imp_tol * X[0]) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) Xn[i] = X[i] + dX[i];
-      if (!imp_residual<F>(P, c, Xn, *Z, Rn, Vn, &Zn)) return false;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        X[i] = Xn[i];
-        R[i] = Rn[i];
-      }
-#pragma unroll
-      for (int k = 0; k < NV; ++k) V[k] = Vn[k];
-      *Z = Zn;
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          Mout[4 * i + j] = ddiv_call((double)J[i][j] - (i == j ? 1.0 : 0.0), c.hdt);
-      if (F::polish(c, X)) imp_polish<F>(P, c, J, X, R, V, Z, dfull);
-      return true;
-    }
-    const double r0 = ((R[0] * R[0] + R[1] * R[1]) + R[2] * R[2]) + R[3] * R[3];
-    double lam = 1.0;
-    int ok = 0;
-    for (int k = 0; k < 10; ++k) {  // at most ten halvings
-#pragma unroll
-      for (int i = 0; i < 4; ++i) Xn[i] = X[i] + dX[i];
-      if (imp_residual<F>(P, c, Xn, *Z, Rn, Vn, &Zn)) {
-        const double r1 = ((Rn[0] * Rn[0] + Rn[1] * Rn[1]) + Rn[2] * Rn[2]) + Rn[3] * Rn[3];
-        if (r1 <= (1.0 - 1e-4 * lam) * r0) {
-          ok = 1;
-          break;
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) dX[i] = 0.5 * dX[i];
-      lam = 0.5 * lam;
-      if (first && k == 3) break;
-    }
-    if (!ok) {
-      if (!fresh_fd) {
-        need_fd = 1;
-        continue;
-      }
-      return false;
-    }
-    double dmax = 0.0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const double dd = fabs(dX[i]);
-      if (dd > dmax) dmax = dd;
-    }
-    broyden(J, dX, R, Rn);
-    fresh_fd = 0;
-    first = 0;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      X[i] = Xn[i];
-      R[i] = Rn[i];
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) V[k] = Vn[k];
-    *Z = Zn;
-    if (prev >= 0.0 && dmax > 0.5 * prev) need_fd = 1;
-    prev = dmax;
-  }
-  return false;
-}
-
-constexpr int IMP_LADDER = 6;  // continuation fallback starts at h / 2^6
+constexpr int IMP_LADDER_RUNGS = 6;  // continuation fallback starts at h / 2^6
 
 // The same residual as a function of the matter primitives Y = (p, u^i):
 // rho = D/W, W = sqrt(1 + u.u), v = u/W, B fixed, X = (tau_t - tau_e(Y), S_t - S(Y)).
@@ -650,169 +474,6 @@ static __device__ __noinline__ bool imp_residual_m(const Params& P, const ImpCel
 #pragma unroll
   for (int i = 0; i < 4; ++i) R[i] = (X[i] - c.Xs[i]) + c.hdt * G[i];
   return true;
-}
-
-// Newton's method on R(Y) = 0 from Y: forward-difference Jacobian at every iterate
-// (steps 1e-7 of the scales p and 1 + |u|), backtracking on |R|^2; converged when
-// every component of the full step is <= 100 imp_tol times its scale (R keeps the
-// rounding of the radiation-sized terms, which the Jacobian carries into Y).
-static __device__ __noinline__ bool imp_newton_m(const Params& P, const ImpCell& c, double* Y,
-                                                 double* X, double* V) {
-  double R[4];
-  if (!imp_residual_m(P, c, Y, R, X, V)) return false;
-  for (int m = 1; m <= P.imp_maxit; ++m) {
-    const double su = 1.0 + dsqrt((Y[1] * Y[1] + Y[2] * Y[2]) + Y[3] * Y[3]);
-    const double sc[4] = {Y[0], su, su, su};
-    double J[4][4];
-    for (int j = 0; j < 4; ++j) {
-      double Yp[4] = {Y[0], Y[1], Y[2], Y[3]};
-      double Rp[4], Xp[4], Vp[NV];
-      Yp[j] = Y[j] + 1e-7 * sc[j];
-      if (!imp_residual_m(P, c, Yp, Rp, Xp, Vp)) {
-        Yp[j] = Y[j] - 1e-7 * sc[j];
-        if (!imp_residual_m(P, c, Yp, Rp, Xp, Vp)) return false;
-      }
-      const double dYj = Yp[j] - Y[j];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) J[i][j] = ddiv_call(Rp[i] - R[i], dYj);
-    }
-    double b[4], dY[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) b[i] = -R[i];
-    if (!solve4(J, b, dY)) return false;
-    bool conv = true;
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      if (fabs(dY[i]) > (100.0 * P.imp_tol) * sc[i]) conv = false;
-    double Yn[4], Rn[4], Xn[4], Vn[NV];
-    if (conv) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) Yn[i] = Y[i] + dY[i];
-      if (!imp_residual_m(P, c, Yn, Rn, Xn, Vn)) return false;
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        Y[i] = Yn[i];
-        X[i] = Xn[i];
-      }
-#pragma unroll
-      for (int k = 0; k < NV; ++k) V[k] = Vn[k];
-      return true;
-    }
-    const double r0 = ((R[0] * R[0] + R[1] * R[1]) + R[2] * R[2]) + R[3] * R[3];
-    double lam = 1.0;
-    bool ok = false;
-    for (int k = 0; k < 40; ++k) {
-#pragma unroll
-      for (int i = 0; i < 4; ++i) Yn[i] = Y[i] + dY[i];
-      if (imp_residual_m(P, c, Yn, Rn, Xn, Vn)) {
-        const double r1 = ((Rn[0] * Rn[0] + Rn[1] * Rn[1]) + Rn[2] * Rn[2]) + Rn[3] * Rn[3];
-        if (r1 <= (1.0 - 1e-4 * lam) * r0) {
-          ok = true;
-          break;
-        }
-      }
-#pragma unroll
-      for (int i = 0; i < 4; ++i) dY[i] = 0.5 * dY[i];
-      lam = 0.5 * lam;
-    }
-    if (!ok) return false;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      Y[i] = Yn[i];
-      R[i] = Rn[i];
-      X[i] = Xn[i];
-    }
-#pragma unroll
-    for (int k = 0; k < NV; ++k) V[k] = Vn[k];
-  }
-  return false;
-}
-
-// The matter-primitive solve from the matter state of U* (primitives Vs).
-__device__ __forceinline__ bool solve_matter(const Params& P, const ImpCell& c, const double* Vs,
-                                             double* X, double* V) {
-  const double v2 = (Vs[1] * Vs[1] + Vs[2] * Vs[2]) + Vs[3] * Vs[3];
-  const double W = ddiv(1.0, dsqrt(1.0 - v2));
-  double Y[4] = {Vs[4], W * Vs[1], W * Vs[2], W * Vs[3]};
-  return imp_newton_m(P, c, Y, X, V);
-}
-
-// Implicit step of one cell (Sec. 3.3).  Writes U and V on success; returns a Status.
-// jc (may be null): the cell's Jacobian cache, M = (J - I)/h of its last converged
-// solve (16 entries) and a flag jc[16]; with flag 1 M replaces C^(m) as the first
-// matrix, and the converged matrix is stored back (cleared on failure).  Flag 2: the
-// last solve needed the matter primitives, and the next one starts there.  Order:
-// [flag 2: matter solve]; iteration on X; continuation in h on X; matter solve
-// (unless it was the first attempt).
-template <class F = FormF64>
-__device__ __forceinline__ int implicit_cell(const Params& P, double kappa, double sigma,
-                                             double hdt, const double* Us, double Zguess,
-                                             double* U, double* V, double* jc = nullptr) {
-  if ((kappa == 0.0 && sigma == 0.0) || hdt == 0.0) {
-#pragma unroll
-    for (int k = 0; k < NV; ++k) U[k] = Us[k];
-    return con2prim(P, Us, Zguess, V, nullptr);
-  }
-  ImpCell c;
-  c.kappa = kappa;
-  c.sigma = sigma;
-  c.hdt = hdt;
-  c.D = Us[0];
-  c.taut = Us[4] + Us[8];
-#pragma unroll
-  for (int j = 0; j < 3; ++j) {
-    c.St[j] = Us[1 + j] + Us[9 + j];
-    c.B[j] = Us[5 + j];
-  }
-#pragma unroll
-  for (int i = 0; i < 4; ++i) c.Xs[i] = Us[8 + i];
-  double X[4] = {c.Xs[0], c.Xs[1], c.Xs[2], c.Xs[3]};
-  double R[4], Z = Zguess;
-  // no admissible matter state at X*: the explicit update U* itself is inadmissible
-  if constexpr (F::kReuseW) c.iD = ddiv_call(1.0, c.D);
-  if (!imp_residual<F>(P, c, X, Zguess, R, V, &Z)) return ST_C2P;
-  double Mnew[16], Vs[NV];
-#pragma unroll
-  for (int k = 0; k < NV; ++k) Vs[k] = V[k];
-  const bool tried_m = jc && jc[16] == 2.0;
-  if (tried_m) {
-    if (solve_matter(P, c, Vs, X, V)) {
-      matter_state(c, X, U);
-      return ST_OK;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) X[i] = c.Xs[i];
-#pragma unroll
-    for (int k = 0; k < NV; ++k) V[k] = Vs[k];
-    Z = Zguess;
-    imp_residual<F>(P, c, X, Z, R, V, &Z);
-  }
-  bool ok = imp_newton<F>(P, c, X, R, V, &Z, (jc && jc[16] == 1.0) ? jc : nullptr, Mnew);
-  if (!ok) {
-#pragma unroll
-    for (int i = 0; i < 4; ++i) X[i] = c.Xs[i];
-    Z = Zguess;
-    ok = true;
-    for (int j = IMP_LADDER; j >= 0 && ok; --j) {
-      c.hdt = hdt / (double)(1 << j);
-      ok = imp_residual<F>(P, c, X, Z, R, V, &Z);
-      if (ok) ok = imp_newton<F>(P, c, X, R, V, &Z, nullptr, Mnew);
-    }
-    c.hdt = hdt;
-  }
-  bool matter = false;
-  if (!ok && !tried_m) {
-    ok = solve_matter(P, c, Vs, X, V);
-    matter = ok;
-  }
-  if (jc) {
-#pragma unroll
-    for (int k = 0; k < 16; ++k) jc[k] = (ok && !matter) ? Mnew[k] : 0.0;
-    jc[16] = ok ? (matter ? 2.0 : 1.0) : 0.0;
-  }
-  if (!ok) return ST_IMPLICIT;
-  matter_state(c, X, U);
-  return ST_OK;
 }
 
 }  // namespace rr
