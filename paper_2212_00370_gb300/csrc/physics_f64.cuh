@@ -146,6 +146,12 @@ __device__ __forceinline__ void prim2con_t(const Params& P, const double* V, dou
   for (int k = 5; k < NV; ++k) U[k] = V[k];
 }
 
+// a / b inline, or the shared copy
+template <bool INL>
+__device__ __forceinline__ double cdiv(double a, double b) {
+  return INL ? ddiv(a, b) : ddiv_call(a, b);
+}
+
 // ------------------------------------------------------------- M1 closure
 // xi(f) = (3 + 4f^2)/(5 + 2 sqrt(4 - 3f^2)), P = [(1-xi)/2 delta + (3xi-1)/2 n n] E
 // (Sec. 2.2, Eq. xi); f clamped to 1; no n n term when F_r = 0.
@@ -153,18 +159,20 @@ struct M1 {
   double a, c;  // P_ij = c F_i F_j (+ a on the diagonal)
 };
 
-template <bool SOFT = false>
+// INL: quotients and root inline (the faces), else the shared ones (the cell solver).
+template <bool SOFT = false, bool INL = true>
 __device__ __forceinline__ M1 m1_coef(double E, double Fx, double Fy, double Fz) {
 #ifndef RR_DIV_CALLS
   // factors 2, 4 and 1/2 folded into multiply-adds (their products are exact)
   const double F2 = (mul<SOFT>(Fx, Fx) + mul<SOFT>(Fy, Fy)) + mul<SOFT>(Fz, Fz);
-  double f2 = ddiv(F2, mul<SOFT>(E, E));
+  double f2 = cdiv<INL>(F2, mul<SOFT>(E, E));
   if (fpi::gt_nonneg(f2, 1.0)) f2 = 1.0;
-  const double xi = ddiv(__fma_rn(4.0, f2, 3.0), __fma_rn(2.0, dsqrt(4.0 - mul<SOFT>(3.0, f2)), 5.0));
+  const double r = 4.0 - mul<SOFT>(3.0, f2);
+  const double xi = cdiv<INL>(__fma_rn(4.0, f2, 3.0), __fma_rn(2.0, (INL ? dsqrt(r) : dsqrt_call(r)), 5.0));
   M1 m;
   m.a = mul<SOFT>(__fma_rn(-0.5, xi, 0.5), E);
   const bool z = !fpi::pos(F2);
-  const double mc = ddiv(mul<SOFT>(__fma_rn(0.5, mul<SOFT>(3.0, xi), -0.5), E), z ? 1.0 : F2);
+  const double mc = cdiv<INL>(mul<SOFT>(__fma_rn(0.5, mul<SOFT>(3.0, xi), -0.5), E), z ? 1.0 : F2);
   m.c = z ? 0.0 : mc;
   return m;
 #else
@@ -293,7 +301,7 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
   double xt = x, dx = 0.0, bad = 0.0;
   int it = 0, k = 0;
   bool bound = false;
-  const bool window = !FAST && c2p_window(c);
+  const bool window = SOFT && c2p_window(c);
   const bool zB = lo_hi_zero(c.B2), zSB = lo_hi_zero(c.SB2);
   for (;;) {
     bool ok = gt_nonneg(xt, bad);
@@ -309,8 +317,8 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
         iZ2 = iZ * iZ;
         v2 = (c.S2 + c.SB2 * ((2.0 * Z + c.B2) * iZ2)) * (iZB * iZB);
       } else {
-        iZ = ddiv(1.0, Z);
-        iZB = ddiv(1.0, ZB);
+        iZ = cdiv<SOFT>(1.0, Z);
+        iZB = cdiv<SOFT>(1.0, ZB);
         if (in) {
           const double u = __fma_rn(2.0, Z, c.B2);
           iZ2 = pm<SOFT>(false, iZ, iZ);
@@ -339,6 +347,17 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
         xt = 2.0 * xt;
       } else {
         dx = 0.5 * dx;
+        // halvings that cannot suffice, at once: while |dx| >= 2^(g+2), g the exponent of
+        // x - bad, x + dx lies below bad
+        const uint32_t ed = hi_word(dx) >> 20, eg = hi_word(x - bad) >> 20;
+        if (ed - 0x801u < 0x7feu && eg - 1u < 0x7feu) {  // dx negative, both normal
+          int n = (int)(ed - 0x800u) - (int)eg - 1;
+          if (n > 60 - k) n = 60 - k;
+          if (n > 0) {
+            dx = make(hi_word(dx) - ((uint32_t)n << 20), lo_word(dx));
+            k += n;
+          }
+        }
         xt = x + dx;
       }
       continue;
@@ -352,8 +371,8 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
       p = c.gm1g * (x * omv2 - c.D * ddiv(v2, W + 1.0));
       conv = mag_le(dx, 1e-10 * x);
     } else {
-      W = ddiv(1.0, dsqrt(omv2));
-      const double q = ddiv(v2, W + 1.0);
+      W = cdiv<SOFT>(1.0, SOFT ? dsqrt(omv2) : dsqrt_call(omv2));
+      const double q = cdiv<SOFT>(v2, W + 1.0);
       double tol;
       if (in) {
         const double t = pm<SOFT>(false, x, omv2) - pm<SOFT>(false, c.D, q);
@@ -406,7 +425,7 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
         const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
         df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * iZ3;
       }
-      dx = ddiv(-f, df);
+      dx = cdiv<SOFT>(-f, df);
     }
     xt = x + dx;
     ++it;
@@ -424,7 +443,8 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
 // of the FP64 instructions less per recovery (1 M C1 states: 825 -> 447 us), but a longer
 // chain (a product is ~100 clocks instead of 64) and 20 KB of code: the faces, whose warps
 // run in step, and the recovery itself take it; the cell solver, paced by its slowest cells
-// and its instruction fetches, does not.
+// and its instruction fetches, does not, and calls the shared quotient and root (inline ones
+// cost 3-5 % there: 3D box 89.3 -> 84.8 ms per step with calls here and in the residual).
 template <bool FAST = false, bool SOFT = false>
 static __device__ __noinline__ int con2prim(const Params& P, const double* U, double Zguess,
                                             double* V, double* Zout, double* Wout = nullptr) {
