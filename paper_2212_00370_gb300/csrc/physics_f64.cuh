@@ -100,15 +100,17 @@ struct Aux {
   double v2, iW, W, vB, B2, b0, b[3], bsq, rhoh, ptot;
 };
 
+// B2 (may be null): |B|^2 of the state, where the caller has it.
 template <bool SOFT = false>
-__device__ __forceinline__ void aux_of(const Params& P, const double* V, Aux& a) {
+__device__ __forceinline__ void aux_of(const Params& P, const double* V, Aux& a,
+                                       const double* B2 = nullptr) {
   const double vx = V[1], vy = V[2], vz = V[3];
   const double Bx = V[5], By = V[6], Bz = V[7];
   a.v2 = (mul<SOFT>(vx, vx) + mul<SOFT>(vy, vy)) + mul<SOFT>(vz, vz);
   a.iW = dsqrt(1.0 - a.v2);
   a.W = ddiv(1.0, a.iW);
   a.vB = (mul<SOFT>(vx, Bx) + mul<SOFT>(vy, By)) + mul<SOFT>(vz, Bz);
-  a.B2 = (mul<SOFT>(Bx, Bx) + mul<SOFT>(By, By)) + mul<SOFT>(Bz, Bz);
+  a.B2 = B2 ? *B2 : (mul<SOFT>(Bx, Bx) + mul<SOFT>(By, By)) + mul<SOFT>(Bz, Bz);
   a.b0 = mul<SOFT>(a.W, a.vB);
   a.b[0] = mul<SOFT>(Bx, a.iW) + mul<SOFT>(vx, a.b0);
   a.b[1] = mul<SOFT>(By, a.iW) + mul<SOFT>(vy, a.b0);
@@ -216,10 +218,11 @@ __device__ __forceinline__ void eddington(double E, const double* F, double Dr[3
 //   momentum  S^j v^d - b^j B^d/W + p* delta^{dj}
 //   energy    (tau_e + p*) v^d - b^0 B^d/W
 //   induction v^d B^j - B^d v^j;  radiation F^d, P^{dj}.
+// B2 as in aux_of.
 __device__ __forceinline__ void flux(const Params& P, int d, const double* V, const double* U,
-                                     double* F) {
+                                     double* F, const double* B2 = nullptr) {
   Aux a;
-  aux_of(P, V, a);
+  aux_of(P, V, a, B2);
   const double vd = V[1 + d];
   const double Bd = V[5 + d];
   const double BdW = Bd * a.iW;
@@ -233,8 +236,8 @@ __device__ __forceinline__ void flux(const Params& P, int d, const double* V, co
 #pragma unroll
   for (int j = 0; j < 3; ++j) F[5 + j] = (j == d) ? 0.0 : vd * V[5 + j] - Bd * V[1 + j];
   F[8] = V[9 + d];
-  const M1 m = m1_coef(V[8], V[9], V[10], V[11]);
   const double* Fr = V + 9;
+  const M1 m = m1_coef(V[8], V[9], V[10], V[11]);
 #pragma unroll
   for (int j = 0; j < 3; ++j) F[9 + j] = m1_P(m, Fr, d, j);
 }
@@ -433,8 +436,8 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
   }
 }
 
-// Returns a Status; V, *Zout and *Wout (the Lorentz factor; may be null) are written
-// only on success.
+// Returns a Status; V, *Zout, *Wout (the Lorentz factor) and *B2out (|B|^2; all may be null)
+// are written only on success.
 // Stopping rule: the iteration stops at the Newton step with |dx| <= 1e-10 x (the
 // step is taken).  In Newton's quadratic regime the error left is of order
 // (1e-10 x)^2 / x, below rounding, so the PVM's finite-difference products, which
@@ -447,7 +450,8 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
 // cost 3-5 % there: 3D box 89.3 -> 84.8 ms per step with calls here and in the residual).
 template <bool FAST = false, bool SOFT = false>
 static __device__ __noinline__ int con2prim(const Params& P, const double* U, double Zguess,
-                                            double* V, double* Zout, double* Wout = nullptr) {
+                                            double* V, double* Zout, double* Wout = nullptr,
+                                            double* B2out = nullptr) {
   C2PIn c;
   c.D = U[0];
   c.S[0] = U[1];
@@ -479,6 +483,7 @@ static __device__ __noinline__ int con2prim(const Params& P, const double* U, do
   for (int k = 5; k < NV; ++k) V[k] = U[k];
   if (Zout) *Zout = e.Z;
   if (Wout) *Wout = e.W;
+  if (B2out) *B2out = c.B2;
   return ST_OK;
 }
 

@@ -642,7 +642,10 @@ __global__ void k_end_step(Batch b) {
   if (b.st.status[i] == 0 && b.st.dt[i] > 0.0) b.st.t[i] = b.st.t[i] + b.st.dt[i];
 }
 
-__global__ void k_prim2con(Params P, const double* __restrict__ V, double* __restrict__ U,
+// The pointwise kernels are bound by integer issue with long chains, so registers are capped
+// for 32 warps per SM: 8 M prim2con 576 -> 537 us, 2 M con2prim 875 -> 828 us (24 and 40 warps:
+// 539, 553 and 844, 847).
+__global__ void __launch_bounds__(256, 4) k_prim2con(Params P, const double* __restrict__ V, double* __restrict__ U,
                            int64_t n) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;
@@ -665,7 +668,7 @@ __global__ void k_prim_Z(Params P, const double* __restrict__ V, double* __restr
   Z[c] = prim_Z(P, v);
 }
 
-__global__ void k_con2prim(Params P, const double* __restrict__ U, const double* __restrict__ Zg,
+__global__ void __launch_bounds__(128, 8) k_con2prim(Params P, const double* __restrict__ U, const double* __restrict__ Zg,
                            double* __restrict__ V, int32_t* __restrict__ status, int64_t n) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (c >= n) return;

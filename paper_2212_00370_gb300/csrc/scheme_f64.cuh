@@ -129,12 +129,12 @@ __device__ __forceinline__ int pvm_flux(const Params& P, int d, const double* VL
 #pragma unroll
         for (int k = 0; k < NV; ++k) Ue[k] = Um[k] + Y[k];
       }
-      double Z;
-      if (con2prim<false, true>(P, Ue, j == 0 ? Zg : Zm, Ve, &Z) != ST_OK) {
+      double Z, B2;
+      if (con2prim<false, true>(P, Ue, j == 0 ? Zg : Zm, Ve, &Z, nullptr, &B2) != ST_OK) {
         fail = 1;
         break;
       }
-      flux(P, d, Ve, Ue, Fe);
+      flux(P, d, Ve, Ue, Fe, &B2);
       if (j == 0) {
         Zm = Z;
 #pragma unroll
