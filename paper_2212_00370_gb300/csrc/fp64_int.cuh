@@ -221,6 +221,20 @@ RR_HD double mul_fast(double a, double b) {
   return make((uint32_t)(z >> 32) | ((ahi ^ bhi) & 0x80000000u), (uint32_t)z);
 }
 
+// x as a float, rounded to nearest even, for 2^-126 <= |x| < 2^127 or zero.
+RR_HD float to_float_fast(double x) {
+  const uint32_t hi = hi_word(x), lo = lo_word(x);
+  const uint32_t m = shl_hi(hi & 0x7fffffffu, lo, 3) - (896u << 23);
+  const uint32_t up = (uint32_t)(((uint64_t)(lo << 3) + (0x7fffffffu + (m & 1u))) >> 32);
+  const bool zero = ((hi & 0x7fffffffu) | lo) == 0u;
+  return as_float((zero ? 0u : m + up) | (hi & 0x80000000u));
+}
+// a normal float or zero as a double
+RR_HD double to_double_fast(float f) {
+  const uint32_t u = float_bits(f), m = u & 0x7fffffffu;
+  return make((u & 0x80000000u) | (m ? (m >> 3) + (896u << 20) : 0u), m << 29);
+}
+
 // Comparisons on the bits (an FP64 comparison takes the FP64 pipe like a product).
 RR_HD uint64_t bits(double x) { return ((uint64_t)hi_word(x) << 32) | lo_word(x); }
 constexpr uint64_t kInf = 0x7ff0000000000000ull;
@@ -260,6 +274,18 @@ __device__ __forceinline__ double div(double a, double b) {
       : "+d"(q)
       : "r"((int)plain), "d"(a), "d"(b));
   return q;
+}
+
+// (float)x and (double)f: a conversion takes the FP64 pipe like a product.  The instruction
+// stays for the rest of the range, behind a call (a branch that is not turned into predicates).
+static __device__ __noinline__ float to_float_slow(double x) { return (float)x; }
+static __device__ __noinline__ double to_double_slow(float f) { return (double)f; }
+__device__ __forceinline__ float to_float(double x) {
+  return in_window_or_zero(x, 897, 253) ? to_float_fast(x) : to_float_slow(x);
+}
+__device__ __forceinline__ double to_double(float f) {
+  const uint32_t m = float_bits(f) & 0x7fffffffu;
+  return m - 0x00800000u < 0x7f000000u || m == 0u ? to_double_fast(f) : to_double_slow(f);
 }
 
 // sqrt(x).

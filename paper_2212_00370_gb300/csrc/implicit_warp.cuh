@@ -70,14 +70,14 @@ __device__ __forceinline__ void imp_start_newton(ImpTask<F>& t, bool cached) {
     for (int i = 0; i < 4; ++i)
 #pragma unroll
       for (int j = 0; j < 4; ++j)
-        t.J[i][j] = (JT)((i == j ? 1.0 : 0.0) + t.c.hdt * t.jc[4 * i + j]);
+        t.J[i][j] = conv<JT>((i == j ? 1.0 : 0.0) + t.c.hdt * t.jc[4 * i + j]);
   } else {
     double Jd[4][4];
     picard_matrix(t.c, t.X, t.V, Jd);
 #pragma unroll
     for (int i = 0; i < 4; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) t.J[i][j] = (JT)Jd[i][j];
+      for (int j = 0; j < 4; ++j) t.J[i][j] = conv<JT>(Jd[i][j]);
   }
   t.need_fd = false;
   t.fresh_fd = false;
@@ -212,7 +212,7 @@ __device__ __forceinline__ void imp_digest(const Params& P, ImpTask<F>& t, bool 
           if (mt)
             t.Jm[i][j] = q;
           else
-            t.J[i][j] = (JT)q;
+            t.J[i][j] = conv<JT>(q);
         }
         if (j == 3) done = true;
       }
@@ -300,7 +300,7 @@ __device__ __forceinline__ void imp_digest(const Params& P, ImpTask<F>& t, bool 
       imp_take(t, T, R, V, Z);
 #pragma unroll 1
       for (int i = 0; i < 16; ++i)
-        t.Mnew[i] = ddiv_call((double)t.J[i >> 2][i & 3] - ((i >> 2) == (i & 3) ? 1.0 : 0.0), t.c.hdt);
+        t.Mnew[i] = ddiv_call(as_double(t.J[i >> 2][i & 3]) - ((i >> 2) == (i & 3) ? 1.0 : 0.0), t.c.hdt);
       if (F::polish(t.c, t.X)) {
         // Polish: stopping at imp_tol leaves an error of about the last step times the
         // matrix's contraction, which depends on how the iterate was reached.  The iterate

@@ -403,8 +403,8 @@ __device__ __forceinline__ bool c2p_root(const C2PIn& c, double x, int maxit, C2
                          (c.S2 + c.SB2 * (((3.0 * Z + 3.0 * c.B2) * Z + c.B2 * c.B2) * (iZ2 * iZ)));
       const double dp = c.gm1g * (omv2 + dv2 * ((0.5 * c.D) * W - Z));
       const double df = ((1.0 - dp) + (0.5 * c.B2) * dv2) + c.SB2 * (iZ2 * iZ);
-      const float d32 = (float)df;
-      dx = (fabsf(d32) > 1e-30f && fabsf(d32) < 1e30f) ? -f * (double)__frcp_rn(d32) : ddiv(-f, df);
+      const float d32 = to_float(df);
+      dx = (fabsf(d32) > 1e-30f && fabsf(d32) < 1e30f) ? -f * to_double(__frcp_rn(d32)) : ddiv(-f, df);
     } else {
       double f, df;
       const double opv2 = 1.0 + v2;

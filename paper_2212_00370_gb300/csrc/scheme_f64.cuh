@@ -8,20 +8,22 @@
 namespace rr {
 
 // ------------------------------------------------------------ reconstruction
-// Slope limiters of Sec. 3.2 (MinMod, MC, VanLeer); zero slope at extrema.
-__device__ __forceinline__ double limiter(int recon, double dL, double dR) {
+// Half of the limited slope (Sec. 3.2: MinMod, MC, VanLeer); zero at extrema.  The factor 2 of
+// VanLeer's 2 dL dR/(dL + dR) and the half cancel (both are exact).
+__device__ __forceinline__ double half_slope(int recon, double dL, double dR) {
   if (recon == RECON_GODUNOV) return 0.0;
-  if (!(dL * dR > 0.0)) return 0.0;
-  if (recon == RECON_MINMOD) return fabs(dL) < fabs(dR) ? dL : dR;
+  const double p = dL * dR;
+  if (!fpi::pos(p)) return 0.0;
+  if (recon == RECON_MINMOD) return 0.5 * (fabs(dL) < fabs(dR) ? dL : dR);
   if (recon == RECON_MC) {
     double m = 2.0 * fabs(dL);
     const double r = 2.0 * fabs(dR);
     const double c = fabs(0.5 * (dL + dR));
     if (r < m) m = r;
     if (c < m) m = c;
-    return dL > 0.0 ? m : -m;
+    return 0.5 * (dL > 0.0 ? m : -m);
   }
-  return ddiv_call((2.0 * dL) * dR, dL + dR);
+  return ddiv_call(p, dL + dR);
 }
 
 // Face values of the middle cell: vm at its left face, vp at its right face.
@@ -30,9 +32,9 @@ __device__ __forceinline__ void reconstruct(int recon, const double* w0, const d
                                             const double* w2, double* vm, double* vp) {
 #pragma unroll
   for (int k = 0; k < NV; ++k) {
-    const double s = limiter(recon, w1[k] - w0[k], w2[k] - w1[k]);
-    vp[k] = w1[k] + 0.5 * s;
-    vm[k] = w1[k] - 0.5 * s;
+    const double h = half_slope(recon, w1[k] - w0[k], w2[k] - w1[k]);
+    vp[k] = w1[k] + h;
+    vm[k] = w1[k] - h;
   }
   const double v2m = (vm[1] * vm[1] + vm[2] * vm[2]) + vm[3] * vm[3];
   const double F2m = (vm[9] * vm[9] + vm[10] * vm[10]) + vm[11] * vm[11];
@@ -393,19 +395,29 @@ __device__ __forceinline__ void picard_matrix(const ImpCell& c, const double* X,
 // error of ~1e-7 cond(J) is an inexact quasi-Newton step whose error the next FP64
 // residual corrects, as the Broyden matrix's own (larger) error is.
 
+// Conversions between the two on the integer pipes (FP32-bulk form).
+template <class JT>
+__device__ __forceinline__ JT conv(double x);
+template <>
+__device__ __forceinline__ double conv<double>(double x) { return x; }
+template <>
+__device__ __forceinline__ float conv<float>(double x) { return fpi::to_float(x); }
+__device__ __forceinline__ double as_double(double x) { return x; }
+__device__ __forceinline__ double as_double(float x) { return fpi::to_double(x); }
+
 // Newton direction dX = -J^-1 R: solved in JT, returned in double; false if singular.
 template <class JT>
 __device__ __forceinline__ bool newton_dir(const JT J[4][4], const double* R, double* dX) {
   JT A[4][4], b[4], x[4];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    b[i] = (JT)(-R[i]);
+    b[i] = conv<JT>(-R[i]);
 #pragma unroll
     for (int j = 0; j < 4; ++j) A[i][j] = J[i][j];
   }
   if (!solve4(A, b, x)) return false;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) dX[i] = (double)x[i];
+  for (int i = 0; i < 4; ++i) dX[i] = as_double(x[i]);
   return true;
 }
 
@@ -416,11 +428,11 @@ __device__ __forceinline__ void broyden(JT J[4][4], const double* dXd, const dou
                                         const double* Rn) {
   JT dX[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) dX[i] = (JT)dXd[i];
+  for (int i = 0; i < 4; ++i) dX[i] = conv<JT>(dXd[i]);
   const JT s2 = ((dX[0] * dX[0] + dX[1] * dX[1]) + dX[2] * dX[2]) + dX[3] * dX[3];
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
-    const JT dRi = (JT)(Rn[i] - R[i]);
+    const JT dRi = conv<JT>(Rn[i] - R[i]);
     const JT Jd = ((J[i][0] * dX[0] + J[i][1] * dX[1]) + J[i][2] * dX[2]) + J[i][3] * dX[3];
     const JT q = ddiv_call(dRi - Jd, s2);
 #pragma unroll

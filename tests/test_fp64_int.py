@@ -70,6 +70,17 @@ int main(int, char** v) {
     check(mul_fast(c, m), c * m, c, m);                       // and ties: c m with short mantissas
     check(mul_fast(m, m), m * m, m, m);
     check(mul_fast<true>(i % 2 ? c : 0.0 * c, i % 3 ? m : -0.0), (i % 2 ? c : 0.0 * c) * (i % 3 ? m : -0.0), c, m);
+    const double y = from(((897 + g() % 253) << 52) | (i % 2 ? mant(g) : (g() & F) | ((1ull << 29) - 1)) | (g() & (1ull << 63)));
+    check(to_float_fast(y), (float)y, y, 0);
+    check(to_double_fast((float)y), (double)(float)y, y, 0);
+    // comparisons on the bits, with zeros, infinities and NaN of both signs
+    const double sp[8] = {0.0, -0.0, INFINITY, -INFINITY, NAN, -NAN, 1.0, 0x1p-1074};
+    const double u = i % 3 ? a : sp[g() % 8], w2 = i % 5 ? b : sp[g() % 8], n = std::fabs(w2);
+    if (gt_nonneg(u, n) != (u > n) && n == n) check(u, n, 1, 1);
+    if (pos(u) != (u > 0.0)) check(u, 0, 2, 2);
+    if (mag_gt(u, w2) != (std::fabs(u) > std::fabs(w2))) check(u, w2, 3, 3);
+    if (n == n && mag_le(u, n) != (std::fabs(u) <= n)) check(u, n, 4, 4);
+    if (below_one(std::fabs(u)) != (std::fabs(u) < 1.0)) check(u, 1, 5, 5);
     const double s = (m + std::ldexp(1.0, -53)) * m;
     check(sqrt_fast<Seed>(s), std::sqrt(s), s, 0);
   }
