@@ -8,6 +8,9 @@
 // and convergence tests stay FP64).  Same launch structure and lanes as rrmhd_f64.cu.
 #include <cuda_runtime.h>
 
+// This unit is compiled with contraction.  Its quotients and roots are calls (one node in a
+// basic block, like the instruction), its products stay plain: what the compiler fuses, and
+// so every bit of the results, does not depend on how a quotient is formed.
 #define RR_DIV_CALLS
 #include "batch.h"
 #include "batch_index.cuh"

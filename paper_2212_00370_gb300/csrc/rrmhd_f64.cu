@@ -8,11 +8,14 @@
 //             4 cells along the face normal through the boundary map, PLM +
 //             fallback, PVM-int-8 flux -> Fhat.
 //   k_cells : one thread per cell: flux difference and RK combination, then
-//             the implicit radiation-matter solve -> U^(s), V^(s); stage 3 also
-//             reduces the next CFL signal speed per instance.
-// The path is FP64-pipe bound (tens of thousands of FP64 instructions per cell
-// and a few hundred bytes of traffic), so the layout favours full warps and low
-// register pressure over shared-memory staging.
+//             the implicit radiation-matter solve of the warp's cells
+//             (implicit_warp.cuh) -> U^(s), V^(s); stage 3 also reduces the next
+//             CFL signal speed per instance.
+// What bounds them: the FP64 pipe (2 lanes per clock and SM) and, in the cells, the
+// slowest cells.  Quotients, roots, comparisons and the recovery's products of the faces
+// run on the integer pipes (fp64_int.cuh); what is left keeps the pipe 74 % busy in the
+// faces (85 % is what independent FP64 instructions reach) and 64-76 % in the cells while
+// an SM has work.  Traffic is a few hundred bytes per cell, 1-3 % of the HBM rate.
 #include <cuda_runtime.h>
 
 #include "batch.h"
