@@ -65,7 +65,7 @@ struct Params {
 // instructions, 14 clocks per warp and SM against 18.7 on the FP64 pipe, and both pipes run
 // side by side); the factors must be zeros or normal, and the products normal, which the
 // callers' window test ensures.  Same roundings either way.  8 M prim2con: 857 us with FP64
-// products, 537 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
+// products, 503 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
 // take a third of its FP64 instructions away and slow the faces of a Riemann batch by
 // 15-25 % (instruction fetches).
 template <bool SOFT>
@@ -105,16 +105,20 @@ struct Aux {
 };
 
 // B2 (may be null): |B|^2 of the state, where the caller has it.
+// The squares of v and B stay on the FP64 pipe in either form: with all 34 products of
+// prim2con on the integer pipes these hold a warp for ~615 clocks and the FP64 pipe, with the
+// sums alone, for ~410; six products moved back even the two out (8 M prim2con, products
+// moved back: none 537 us, three 529, six 503, nine 503).
 template <bool SOFT = false>
 __device__ __forceinline__ void aux_of(const Params& P, const double* V, Aux& a,
                                        const double* B2 = nullptr) {
   const double vx = V[1], vy = V[2], vz = V[3];
   const double Bx = V[5], By = V[6], Bz = V[7];
-  a.v2 = (mul<SOFT>(vx, vx) + mul<SOFT>(vy, vy)) + mul<SOFT>(vz, vz);
+  a.v2 = (vx * vx + vy * vy) + vz * vz;
   a.iW = dsqrt(1.0 - a.v2);
   a.W = ddiv(1.0, a.iW);
   a.vB = (mul<SOFT>(vx, Bx) + mul<SOFT>(vy, By)) + mul<SOFT>(vz, Bz);
-  a.B2 = B2 ? *B2 : (mul<SOFT>(Bx, Bx) + mul<SOFT>(By, By)) + mul<SOFT>(Bz, Bz);
+  a.B2 = B2 ? *B2 : (Bx * Bx + By * By) + Bz * Bz;
   a.b0 = mul<SOFT>(a.W, a.vB);
   a.b[0] = mul<SOFT>(Bx, a.iW) + mul<SOFT>(vx, a.b0);
   a.b[1] = mul<SOFT>(By, a.iW) + mul<SOFT>(vy, a.b0);

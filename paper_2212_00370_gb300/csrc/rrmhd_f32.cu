@@ -27,10 +27,9 @@ constexpr int kFaceThreads = 128;
 constexpr int kCellThreads = 128;
 
 // Resident warps per SM the cell kernels are compiled for (a register bound of
-// 65536 / (32 x warps) per thread).  12 warps (168 registers; the solver's stack grows
-// from 1.5 to 1.9 KB) hide more of the FP64 dependency latency than the 8 that 255
-// registers allow: +2 % zone-updates/s on C1 in the live step, measured under three
-// cell shapes; 16 warps (128 registers) gained nothing.
+// 65536 / (32 x warps) per thread).  12 warps (168 registers) hide more of the dependency
+// latency than the 8 that 255 registers allow: 4096 Riemann problems, two steps, 177.2 ms at
+// 8 warps, 165.9 at 10, 162.8 at 12, 163.7 at 16; a 2D blast 29.4, 27.6, 28.1, 28.4 ms.
 #ifndef RR_F32_CELL_WARPS
 #define RR_F32_CELL_WARPS 12
 #endif

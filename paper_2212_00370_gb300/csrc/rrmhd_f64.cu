@@ -646,8 +646,8 @@ __global__ void k_end_step(Batch b) {
 }
 
 // The pointwise kernels are bound by integer issue with long chains, so registers are capped
-// for 32 warps per SM: 8 M prim2con 576 -> 537 us, 2 M con2prim 875 -> 828 us (24 and 40 warps:
-// 539, 553 and 844, 847).
+// for 32 warps per SM: 8 M prim2con 576 -> 537 us (503 with the squares back
+// on the FP64 pipe), 2 M con2prim 875 -> 828 us (24 and 40 warps: 539, 553 and 844, 847).
 __global__ void __launch_bounds__(256, 4) k_prim2con(Params P, const double* __restrict__ V, double* __restrict__ U,
                            int64_t n) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
