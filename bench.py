@@ -45,11 +45,11 @@ sys.path.insert(0, ROOT)
 # with ncu on a 2048-instance sample of the same distribution.
 FP64_INST_PER_ZONE = {"fp64": {"faces": 2174.0, "cells": 2616.0},
                       "fp32_bulk": {"faces": 4.0, "cells": 1593.0},
-                      "fp64_tangent": {"faces": 5238.0, "cells": 4591.0}}
+                      "fp64_tangent": {"faces": 4991.0, "cells": 2615.0}}
 # DRAM bytes per cell of one launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)
 TRAFFIC_PER_CELL = {"fp64": {"faces": 583.0, "cells": 1859.0},
                     "fp32_bulk": {"faces": 443.0, "cells": 2593.0},
-                    "fp64_tangent": {"faces": 241.0, "cells": 1669.0}}
+                    "fp64_tangent": {"faces": 772.0, "cells": 1855.0}}
 # Nominal FP64 rate of GB300: 1.25 TFLOP/s = 6.25e11 FP64-pipe instructions/s
 # (2 per SM per clock on 152 SMs at 2.07 GHz).  The roofline divides by the rate
 # rrmhd_probe_fp64 measures in the same run; the nominal figure is reported beside it.
