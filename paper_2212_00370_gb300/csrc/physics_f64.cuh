@@ -65,7 +65,7 @@ struct Params {
 // instructions, 14 clocks per warp and SM against 18.7 on the FP64 pipe, and both pipes run
 // side by side); the factors must be zeros or normal, and the products normal, which the
 // callers' window test ensures.  Same roundings either way.  8 M prim2con: 857 us with FP64
-// products, 503 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
+// products, 510 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
 // take a third of its FP64 instructions away and slow the faces of a Riemann batch by
 // 15-25 % (instruction fetches).
 template <bool SOFT>
@@ -84,17 +84,21 @@ __device__ __forceinline__ double scale_add(double p, double a, double b) {
 #endif
 }
 
-// Window in which the SOFT products of prim2con and prim_Z are valid: |v| from 2^-200 to 1
-// and |B| within 2^+-100, or zeros; rho and p within 2^+-150.  Every product there has at
-// most six factors and every difference keeps at least the last bit of its terms: all of
-// them stay far inside 2^+-1022 or are exact zeros.
+// Window in which the SOFT products of prim2con and prim_Z are valid: |v_k| from 2^-200 to 1
+// and |B_k| within 2^+-100, or zeros; rho and p within 2^+-150; v^2 < 1, so that W is a
+// number in [1, 2^27).  Every product there has at most six factors and every difference
+// keeps at least the last bit of its terms: all of them stay far inside 2^+-1022 or are
+// exact zeros.  v^2 is the sum aux_of forms.  8 M prim2con: 503 us without the test of v^2
+// (and finite numbers where W is not one), 510 with it; 527 with v^2, 1/W and W formed once
+// ahead of the branch, 529 with the test after the products, 509 with a bound of v^2 in FP32
+// first.
 __device__ __forceinline__ bool soft_matter(const double* V) {
   using namespace fpi;
   bool ok = in_window(V[0], 1023 - 150, 300) && in_window(V[4], 1023 - 150, 300);
 #pragma unroll
   for (int k = 1; k < 4; ++k)
     ok = ok && in_window_or_zero(V[k], 1023 - 200, 200) && in_window_or_zero(V[4 + k], 1023 - 100, 200);
-  return ok;
+  return ok && below_one((V[1] * V[1] + V[2] * V[2]) + V[3] * V[3]);
 }
 
 // ---------------------------------------------------------------- aux state
