@@ -65,7 +65,7 @@ struct Params {
 // instructions, 14 clocks per warp and SM against 18.7 on the FP64 pipe, and both pipes run
 // side by side); the factors must be zeros or normal, and the products normal, which the
 // callers' window test ensures.  Same roundings either way.  8 M prim2con: 857 us with FP64
-// products, 510 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
+// products, 482 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
 // take a third of its FP64 instructions away and slow the faces of a Riemann batch by
 // 15-25 % (instruction fetches).
 template <bool SOFT>
@@ -86,15 +86,17 @@ __device__ __forceinline__ double scale_add(double p, double a, double b) {
 
 // Window in which the SOFT products of prim2con and prim_Z are valid: |v_k| from 2^-200 to 1
 // and |B_k| within 2^+-100, or zeros; rho and p within 2^+-150; v^2 < 1, so that W is a
-// number in [1, 2^27).  Every product there has at most six factors and every difference
-// keeps at least the last bit of its terms: all of them stay far inside 2^+-1022 or are
-// exact zeros.  v^2 is the sum aux_of forms.  8 M prim2con: 503 us without the test of v^2
-// (and finite numbers where W is not one), 510 with it; 527 with v^2, 1/W and W formed once
-// ahead of the branch, 529 with the test after the products, 509 with a bound of v^2 in FP32
-// first.
-__device__ __forceinline__ bool soft_matter(const double* V) {
+// number in [1, 2^27); gamma/(gamma-1), which is in [1, 2^52] for a finite gamma and NaN for an
+// infinite one.  Every product there has at most six factors and every difference keeps at
+// least the last bit of its terms: all of them stay far inside 2^+-1022 or are exact zeros.  v^2
+// is the sum aux_of forms.  8 M prim2con: 503 us without the test of v^2 (and finite numbers
+// where W is not one), 510 with it, 482 with that of gamma as well (another schedule of the
+// same products); with the test of v^2, 527 with v^2, 1/W and W formed once ahead of the branch,
+// 529 with the test after the products, 509 with a bound of v^2 in FP32 first.
+__device__ __forceinline__ bool soft_matter(const Params& P, const double* V) {
   using namespace fpi;
-  bool ok = in_window(V[0], 1023 - 150, 300) && in_window(V[4], 1023 - 150, 300);
+  bool ok = in_window(P.gfac, 1023, 60) && in_window(V[0], 1023 - 150, 300) &&
+            in_window(V[4], 1023 - 150, 300);
 #pragma unroll
   for (int k = 1; k < 4; ++k)
     ok = ok && in_window_or_zero(V[k], 1023 - 200, 200) && in_window_or_zero(V[4 + k], 1023 - 100, 200);
@@ -286,7 +288,8 @@ struct C2PPt {  // the root
 // (the same values to a few ulps) and an inexact Newton step with an FP32 reciprocal of
 // df (~6e-8 relative).
 // Whether the products of the evaluation may be formed by mul_fast: D and S^2 within
-// 2^+-80, B^2 and (S.B)^2 as well or zero.  With x in [2^-400, 2^80) every factor and every
+// 2^+-80, B^2 and (S.B)^2 as well or zero, (gamma-1)/gamma in [2^-60, 2) (NaN for an infinite
+// gamma).  With x in [2^-400, 2^80) every factor and every
 // product of the evaluation is then normal (|h| <= 3/Z, the sums that can cancel to zero
 // are tested where they are used).
 __device__ __forceinline__ bool lo_hi_zero(double x) { return fpi::bits(x) == 0; }
@@ -296,7 +299,7 @@ __device__ __forceinline__ double zsel(bool z, double x) { return z ? 0.0 : x; }
 __device__ __forceinline__ bool c2p_window(const C2PIn& c) {
   using namespace fpi;
   constexpr uint32_t lo = 1023 - 80, n = 160;
-  return in_window(c.D, lo, n) && in_window(c.S2, lo, n) &&
+  return in_window(c.gm1g, 1023 - 60, 61) && in_window(c.D, lo, n) && in_window(c.S2, lo, n) &&
          (in_window(c.B2, lo, n) || lo_hi_zero(c.B2)) &&
          (in_window(c.SB2, lo, n) || lo_hi_zero(c.SB2));
 }

@@ -654,7 +654,7 @@ __global__ void __launch_bounds__(256, 4) k_prim2con(Params P, const double* __r
   if (c >= n) return;
   double v[NV], u[NV];
   load12(V, n, c, v);
-  if (soft_matter(v))
+  if (soft_matter(P, v))
     prim2con_t<true>(P, v, u);
   else
     prim2con_t<false>(P, v, u);

@@ -1,6 +1,6 @@
-"""The windows in which the pointwise conversions take products on the integer pipes keep out
-what makes a factor infinite or NaN: speeds of light and above.  Equal to the oracle bit for
-bit, NaN and infinities included."""
+"""The windows in which the conversions take products on the integer pipes keep out what makes
+a factor infinite or NaN: speeds of light and above, an infinite gamma (gamma/(gamma - 1) and
+its inverse are then NaN).  Equal to the oracle bit for bit, NaN and infinities included."""
 import numpy as np
 import pytest
 
@@ -49,3 +49,29 @@ def test_prim2con_at_the_speed_of_light(field):
     same(ctx.prim2con(Vt).cpu().numpy(), U, "prim2con")
     ctx.set_state(Vt)
     same(ctx.get_state()[0].cpu().numpy(), U, "set_state")
+
+
+@pytest.mark.parametrize("call", ["prim2con", "con2prim"])
+def test_conversions_with_an_infinite_gamma(call):
+    n, gamma = 100000, float("inf")
+    r = np.random.default_rng(12)
+    V = fast_states(n, 12, 1.0)
+    V[1:4] *= r.uniform(0, 1, n)
+    for k in (0, 4, 8):
+        V[k] = 2.0 ** r.uniform(-20, 20, n)
+    V[5:8] *= 2.0 ** r.uniform(-10, 10, n)
+    P = O.Params(gamma=gamma)
+    ctx = rrmhd.Context([rrmhd.make_grid(1, (8,), (0.1,))], gamma=gamma)
+    if call == "prim2con":
+        same(ctx.prim2con(torch.tensor(V, device="cuda")).cpu().numpy(), O.prim2con(V, P), call)
+        return
+    U = O.prim2con(V, O.Params(gamma=4 / 3))
+    ok = np.isfinite(U).all(0)
+    U = np.ascontiguousarray(U[:, ok])
+    for guess in (None, U[0] * 2.0 ** r.uniform(-10, 10, ok.sum())):
+        Vr, _, st = O.con2prim(U, P, guess)
+        g = None if guess is None else torch.tensor(guess, device="cuda")
+        Vg, sg = ctx.con2prim(torch.tensor(U, device="cuda"), g)
+        assert (st != 0).all()          # the pressure is NaN: no state is recovered
+        same(sg.cpu().numpy().astype(float), st.astype(float), "status")
+        same(Vg.cpu().numpy(), np.zeros_like(Vr), "con2prim")
