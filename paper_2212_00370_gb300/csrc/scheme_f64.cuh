@@ -8,8 +8,15 @@
 namespace rr {
 
 // ------------------------------------------------------------ reconstruction
+// Half of VanLeer's slope 2 dL dR/(dL + dR), in that order.
+static __device__ __noinline__ double vanleer_half(double dL, double dR) {
+  return 0.5 * ddiv_call((2.0 * dL) * dR, dL + dR);
+}
+
 // Half of the limited slope (Sec. 3.2: MinMod, MC, VanLeer); zero at extrema.  The factor 2 of
-// VanLeer's 2 dL dR/(dL + dR) and the half cancel (both are exact).
+// VanLeer's slope and the half cancel (both are exact) while dL and dR are within 2^+-500: the
+// product, the sum and the quotient are normal then.  Where dL dR is subnormal, the product
+// with the factor has one bit more.
 __device__ __forceinline__ double half_slope(int recon, double dL, double dR) {
   if (recon == RECON_GODUNOV) return 0.0;
   const double p = dL * dR;
@@ -23,7 +30,8 @@ __device__ __forceinline__ double half_slope(int recon, double dL, double dR) {
     if (c < m) m = c;
     return 0.5 * (dL > 0.0 ? m : -m);
   }
-  return ddiv_call(p, dL + dR);
+  if (fpi::in_window(dL, 523, 1000) && fpi::in_window(dR, 523, 1000)) return ddiv_call(p, dL + dR);
+  return vanleer_half(dL, dR);
 }
 
 // Face values of the middle cell: vm at its left face, vp at its right face.
