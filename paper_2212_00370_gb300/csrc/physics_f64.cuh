@@ -61,11 +61,11 @@ struct Params {
   double gm1g;  // (gamma-1)/gamma
 };
 
-// Products.  SOFT (the pointwise kernels): on the integer pipes (fpi::mul_fast, ~30 integer
-// instructions, 14 clocks per warp and SM against 18.7 on the FP64 pipe, and both pipes run
-// side by side); the factors must be zeros or normal, and the products normal, which the
-// callers' window test ensures.  Same roundings either way.  8 M prim2con: 857 us with FP64
-// products, 482 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
+// Products of prim2con.  SOFT (the pointwise kernel): on the integer pipes (fpi::mul_fast, ~30
+// integer instructions, 14 clocks per warp and SM against 18.7 on the FP64 pipe, and both pipes
+// run side by side); the factors must be zeros or normal, and the products normal, which the
+// caller's window test (soft_matter) ensures.  Same roundings either way.  8 M prim2con: 857 us
+// with FP64 products, 482 with these.  The flux keeps FP64 products: 47 more inline ones (24 KB)
 // take a third of its FP64 instructions away and slow the faces of a Riemann batch by
 // 15-25 % (instruction fetches).
 template <bool SOFT>
@@ -75,7 +75,9 @@ __device__ __forceinline__ double mul(double a, double b) {
   else
     return a * b;
 }
-// b + p a for p a power of two: one rounding either way (p a is exact)
+// b + p a for p a power of two: one rounding either way where p a is exact.  (It is not where
+// it is subnormal: the multiply-add then keeps the bit that the product would round off, and
+// the last bit of a sum next to 2^-1022 may differ from the plain form's.)
 __device__ __forceinline__ double scale_add(double p, double a, double b) {
 #ifdef RR_DIV_CALLS
   return b + p * a;
@@ -84,8 +86,8 @@ __device__ __forceinline__ double scale_add(double p, double a, double b) {
 #endif
 }
 
-// Window in which the SOFT products of prim2con and prim_Z are valid: |v_k| from 2^-200 to 1
-// and |B_k| within 2^+-100, or zeros; rho and p within 2^+-150; v^2 < 1, so that W is a
+// Window in which the SOFT products of prim2con are valid: |v_k| from 2^-200 to 1 and
+// |B_k| within 2^+-100, or zeros; rho and p within 2^+-150; v^2 < 1, so that W is a
 // number in [1, 2^27); gamma/(gamma-1), which is in [1, 2^52] for a finite gamma and NaN for an
 // infinite one.  Every product there has at most six factors and every difference keeps at
 // least the last bit of its terms: all of them stay far inside 2^+-1022 or are exact zeros.  v^2
@@ -135,11 +137,10 @@ __device__ __forceinline__ void aux_of(const Params& P, const double* V, Aux& a,
 }
 
 // rho h W^2: the con2prim unknown Z of a primitive state (warm starts).
-template <bool SOFT>
-__device__ __forceinline__ double prim_Z_t(const Params& P, const double* V) {
+__device__ __forceinline__ double prim_Z(const Params& P, const double* V) {
   Aux a;
-  aux_of<SOFT>(P, V, a);
-  return mul<SOFT>(a.rhoh, mul<SOFT>(a.W, a.W));
+  aux_of(P, V, a);
+  return a.rhoh * (a.W * a.W);
 }
 
 // Eq. eqU, with rho W^2 - rho W = D u^2/(W+1) (u^2 = W^2 v^2).
@@ -161,6 +162,9 @@ __device__ __forceinline__ void prim2con_t(const Params& P, const double* V, dou
 #pragma unroll
   for (int k = 5; k < NV; ++k) U[k] = V[k];
 }
+__device__ __forceinline__ void prim2con(const Params& P, const double* V, double* U) {
+  prim2con_t<false>(P, V, U);
+}
 
 // a / b inline, or the shared copy
 template <bool INL>
@@ -176,19 +180,19 @@ struct M1 {
 };
 
 // INL: quotients and root inline (the faces), else the shared ones (the cell solver).
-template <bool SOFT = false, bool INL = true>
+template <bool INL = true>
 __device__ __forceinline__ M1 m1_coef(double E, double Fx, double Fy, double Fz) {
 #ifndef RR_DIV_CALLS
   // factors 2, 4 and 1/2 folded into multiply-adds (their products are exact)
-  const double F2 = (mul<SOFT>(Fx, Fx) + mul<SOFT>(Fy, Fy)) + mul<SOFT>(Fz, Fz);
-  double f2 = cdiv<INL>(F2, mul<SOFT>(E, E));
+  const double F2 = (Fx * Fx + Fy * Fy) + Fz * Fz;
+  double f2 = cdiv<INL>(F2, E * E);
   if (fpi::gt_nonneg(f2, 1.0)) f2 = 1.0;
-  const double r = 4.0 - mul<SOFT>(3.0, f2);
+  const double r = 4.0 - 3.0 * f2;
   const double xi = cdiv<INL>(__fma_rn(4.0, f2, 3.0), __fma_rn(2.0, (INL ? dsqrt(r) : dsqrt_call(r)), 5.0));
   M1 m;
-  m.a = mul<SOFT>(__fma_rn(-0.5, xi, 0.5), E);
+  m.a = __fma_rn(-0.5, xi, 0.5) * E;
   const bool z = !fpi::pos(F2);
-  const double mc = cdiv<INL>(mul<SOFT>(__fma_rn(0.5, mul<SOFT>(3.0, xi), -0.5), E), z ? 1.0 : F2);
+  const double mc = cdiv<INL>(__fma_rn(0.5, 3.0 * xi, -0.5) * E, z ? 1.0 : F2);
   m.c = z ? 0.0 : mc;
   return m;
 #else
@@ -207,9 +211,8 @@ __device__ __forceinline__ M1 m1_coef(double E, double Fx, double Fy, double Fz)
 #endif
 }
 
-template <bool SOFT = false>
 __device__ __forceinline__ double m1_P(const M1& m, const double* F, int i, int j) {
-  const double t = mul<SOFT>(m.c, mul<SOFT>(F[i], F[j]));
+  const double t = m.c * (F[i] * F[j]);
   return (i == j) ? t + m.a : t;
 }
 
@@ -254,13 +257,6 @@ __device__ __forceinline__ void flux(const Params& P, int d, const double* V, co
   const M1 m = m1_coef(V[8], V[9], V[10], V[11]);
 #pragma unroll
   for (int j = 0; j < 3; ++j) F[9 + j] = m1_P(m, Fr, d, j);
-}
-
-__device__ __forceinline__ double prim_Z(const Params& P, const double* V) {
-  return prim_Z_t<false>(P, V);
-}
-__device__ __forceinline__ void prim2con(const Params& P, const double* V, double* U) {
-  prim2con_t<false>(P, V, U);
 }
 
 // ------------------------------------------------------------- con2prim

@@ -307,7 +307,7 @@ static __device__ __noinline__ bool imp_residual(const Params& P, const ImpCell&
     W = ddiv_call(1.0, dsqrt_call(1.0 - v2));
     T = ddiv_call(V[4], V[0]);
   }
-  const M1 m = m1_coef<false, false>(X[0], X[1], X[2], X[3]);
+  const M1 m = m1_coef<false>(X[0], X[1], X[2], X[3]);
   const double u[3] = {W * V[1], W * V[2], W * V[3]};
   const double BP = P.a_rad * ((T * T) * (T * T));
   double Pr[3][3];
@@ -483,7 +483,7 @@ static __device__ __noinline__ bool imp_residual_m(const Params& P, const ImpCel
   for (int i = 0; i < 4; ++i) V[8 + i] = X[i];
   const double T = ddiv_call(Y[0], V[0]);
   const double BP = P.a_rad * ((T * T) * (T * T));
-  const M1 m = m1_coef<false, false>(X[0], X[1], X[2], X[3]);
+  const M1 m = m1_coef<false>(X[0], X[1], X[2], X[3]);
   double Pr[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
