@@ -13,9 +13,12 @@
 //             CFL signal speed per instance.
 // What bounds them: the FP64 pipe (2 lanes per clock and SM) and, in the cells, the
 // slowest cells.  Quotients, roots, comparisons and the recovery's products of the faces
-// run on the integer pipes (fp64_int.cuh); what is left keeps the pipe 74 % busy in the
-// faces (85 % is what independent FP64 instructions reach) and 64-76 % in the cells while
-// an SM has work.  Traffic is a few hundred bytes per cell, 1-3 % of the HBM rate.
+// run on the integer pipes (fp64_int.cuh); what is left keeps the pipe 70 % busy in the
+// faces (85 % is what independent FP64 instructions reach) and 72-73 % in the cells while
+// an SM has work, 61-71 % over a launch.  Traffic of a Riemann batch: 583 B per cell and
+// launch in the faces (0.12 TB/s, 2 % of the copy rate), 1.8-1.9 KB in the cells (0.2-0.34
+// TB/s, 3-5 %), of which some 700 B are state and the rest the solver's stack (2.1 KB per
+// thread).
 #include <cuda_runtime.h>
 
 #include "batch.h"
@@ -36,7 +39,9 @@ constexpr int kCellThreads = 128;
 // thread, 8 warps per SM); W > 0 asks for W warps per SM in blocks of BS threads (at
 // most 32 resident blocks per SM).  Faces: with the quotients and the recovery's products
 // on the integer pipes the FP64 pipe is no longer kept busy by 8 warps (flux sweep of
-// 513 x 767: 2.10 ms at 8, 1.90 at 12, 1.96 at 16; 3D box step 90.8, 86.3, 87.2 ms).
+// 513 x 767: 2.10 ms at 8, 1.90 at 12, 1.96 at 16; 3D box step 90.8, 86.3, 87.2 ms; sweep of
+// 1000 Riemann problems 5.99 ms at 8, 5.68 at 12, and 11.34 and 11.31 with tangent products,
+// whose quotients are still on the FP64 pipe: the spills of the tighter bound cost them nothing).
 // Cells: 12 and 16 warps are 2-10 % slower, their spills and instruction fetches cost more.
 #ifndef RR_F64_FACE_WARPS
 #define RR_F64_FACE_WARPS 12
@@ -646,8 +651,8 @@ __global__ void k_end_step(Batch b) {
 }
 
 // The pointwise kernels are bound by integer issue with long chains, so registers are capped
-// for 32 warps per SM: 8 M prim2con 576 -> 537 us (503 with the squares back
-// on the FP64 pipe), 2 M con2prim 875 -> 828 us (24 and 40 warps: 539, 553 and 844, 847).
+// for 32 warps per SM: 8 M prim2con 576 -> 537 us (later steps: 482), 2 M con2prim 875 -> 828 us
+// (24 and 40 warps: 539, 553 and 844, 847).
 __global__ void __launch_bounds__(256, 4) k_prim2con(Params P, const double* __restrict__ V, double* __restrict__ U,
                            int64_t n) {
   const int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;

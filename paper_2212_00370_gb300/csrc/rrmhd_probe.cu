@@ -1,7 +1,7 @@
 // rrmhd_probe.cu -- throughput probe of the FP64 pipe.
 //
 // The path's cell and face kernels are bound by the FP64 pipe (no dense
-// contraction, and HBM under 1 % busy), so their roofline denominator is the rate
+// contraction, and HBM 3-12 % busy), so their roofline denominator is the rate
 // at which this GPU retires FP64 instructions.  This probe measures it: every
 // thread runs eight independent chains of DFMA (so the pipe, not the ~latency of
 // one chain, is the limit), 64 warps per SM on every SM, timed with CUDA events on

@@ -377,9 +377,12 @@ bool step(rrmhd_server* s, std::vector<rrmhd_result>& finished, int64_t& zone_up
   SRV_CUDA(s, cudaMemcpyAsync(s->h_status, s->B.status, sizeof(int) * n, cudaMemcpyDeviceToHost, st));
   SRV_CUDA(s, cudaMemcpyAsync(s->h_smax, s->B.smax, sizeof(unsigned long long) * n,
                               cudaMemcpyDeviceToHost, st));
-  // The engine thread sleeps through the step instead of spinning on a core: 0.11 ms a step
-  // (a mix of small requests 0.65 -> 0.76 ms, 20 requests of up to 256^2 cells 75 -> 78 ms in
-  // all) for a host core left to the callers.
+  // The engine thread sleeps through the step instead of spinning on a core.  That leaves the
+  // core to the callers and costs the wake-up: 18 small FP32-bulk requests 0.70 -> 0.77 ms per
+  // step, 20 of up to 256^2 cells 66.5 -> 68.9 ms in all.  It also decides how soon a short
+  // request is done: one of 150 steps that is joined by others 50 and 100 ms after it takes
+  // 113-119 ms, and 98 ms spinning, when the last ones no longer meet it (the continuous-batching
+  // test asks that they do).
   SRV_CUDA(s, cudaEventRecord(s->stepped, st));
   SRV_CUDA(s, cudaEventSynchronize(s->stepped));
 

